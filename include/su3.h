@@ -66,12 +66,19 @@ typedef enum { SU3_REPR_FULL18 = 0, SU3_REPR_TWOROW12 = 1 } su3_repr;
 typedef enum { SU3_LAYOUT_AOS = 0, SU3_LAYOUT_AOSOA32 = 1, SU3_LAYOUT_SOA = 2 } su3_layout;
 
 /*
- * Arithmetic of the F64 storage type. NATIVE: FP64 fused multiply-adds (the plain method).
+ * Arithmetic of the F64 storage type. NATIVE: FP64 accuracy (the plain method's results). a x b
+ * is computed by FP64 fused multiply-adds and, beside them, in 61-bit fixed point on the integer
+ * units with one rounding per result: off by at most half an ulp + 5 * 2^-58 of (the largest real
+ * of the row of a) x (the largest real of b[j]), each rounded up to a power of two, for rows and
+ * matrices whose reals are of similar size; the others (zeros, reals spread over many binary
+ * orders, extreme or non-finite values) by FP64 FMAs throughout. On random SU(3) matrices that is
+ * half the error of FP64 FMAs alone.
  * F32PAIR: FP64 storage, arithmetic on unevaluated pairs of FP32 numbers. Each a element is split
  * into hi + lo with integer operations; each output real is a compensated dot product (TwoSum on
  * the running FP32 sum, the product error and the product's share of the TwoSum error added by one
  * FMA, error terms accumulated in a second FP32 number) and becomes FP64 with one FP64 add.
- * GB300's FP64 units run at 1/64 of its FP32 rate, so this is several times faster. Accuracy: about 2^-45 times
+ * GB300's FP64 units run at 1/64 of its FP32 rate, so this is several times faster than FP64 FMAs
+ * (and somewhat faster than NATIVE). Accuracy: about 2^-45 times
  * sum_m |a[k][m]||b[m][l]| per output (measured max 3.3e-14 against the FP64 oracle on SU(3)
  * data, whose entries are <= 1). Valid for finite inputs with |x| < 2^127; input magnitudes below
  * 2^-74 (including zeros) act as values below 2^-73. All repr pairs are supported; for

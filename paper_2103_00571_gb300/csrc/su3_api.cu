@@ -844,10 +844,7 @@ static su3_status fill_batch(su3_handle* h, int32_t n, const su3_batch_item* ite
     o.n_sites = d.n_sites;
     o.dtype = d.dtype;
     o.first_tile = tiles;
-    o.arith = d.arith;
-    o.reserved = 0;
-    memcpy(o.b, it.b, sizeof(o.b));
-    split_b_pairs(&it.b[0][0][0][0], o.bpair);
+    fill_batch_b(&o, d.dtype, d.arith, &it.b[0][0][0][0]);
     const int64_t t = batch_tile_count(d.n_sites, d.dtype, h->bcfg.tile_sites);
     if ((int64_t)tiles + t > (1ll << 30)) return fail(h, SU3_ERR_INVALID_ARG, "batch too large");
     tiles += (int)t;

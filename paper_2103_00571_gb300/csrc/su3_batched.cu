@@ -32,6 +32,7 @@ struct TileInfo {
 
 struct BatchArgs {
   float unit;  // 1.0 for FP32-pair arithmetic (a parameter, so the compiler cannot fold it)
+  FixedConst fixk;  // of the FP64 rows in fixed point (parameters for the same reason)
   const BatchDesc* descs;
   int n;
   int total_tiles;
@@ -86,6 +87,24 @@ __device__ __forceinline__ void batch_tile_compute(unsigned char* in, int nt, co
 #pragma unroll
       for (int l = 0; l < 3; ++l) p[3 * row + l] = S::pack(cre[l], cim[l]);
     }
+  }
+}
+
+// FP64 lattice: rows in fixed point (the op of the single-lattice kernels, so the same bits).
+template <int TPL>
+__device__ __forceinline__ void batch_tile_compute_f64(unsigned char* in, int nt, const BatchDesc& d,
+                                                       const FixedConst& k) {
+  const int j = threadIdx.x & 3;
+  NativeOp<kF64, 9, 3> op;
+  op.init(d.b + 18 * j, 0);
+  op.fix.take(d.bfix[j], d.eb[j], d.fixed ? kFixExpRange : 0, k);
+  const int links = 4 * nt;
+  for (int q = threadIdx.x; q < TPL * links; q += blockDim.x) {
+    int row, link;
+    batch_item<TPL>(q, links, row, link);
+    double2* p = reinterpret_cast<double2*>(in + (size_t)link * 144);
+    if constexpr (TPL == 1) op.apply(p, p);
+    else op.apply_row(p, p, row);
   }
 }
 
@@ -170,7 +189,7 @@ __global__ void __launch_bounds__(256) su3_batched_kernel(const __grid_constant_
     if (ok) {
       if (dtype == SU3_F64) {
         if (d.arith == SU3_ARITH_F32PAIR) batch_tile_compute_pair<TPL>(in, ti.nt, d, p.unit);
-        else batch_tile_compute<kF64, TPL>(in, ti.nt, d);
+        else batch_tile_compute_f64<TPL>(in, ti.nt, d, p.fixk);
       } else {
         batch_tile_compute<kF32, TPL>(in, ti.nt, d);
       }
@@ -244,6 +263,7 @@ su3_status launch_batched(const BatchDesc* descs_dev, int n, int total_tiles, co
   if (total_tiles == 0) return SU3_OK;
   BatchArgs p;
   p.unit = 1.0f;
+  p.fixk = fixed_const();
   p.descs = descs_dev;
   p.n = n;
   p.total_tiles = total_tiles;
@@ -380,10 +400,7 @@ static su3_status mult_batched_static_impl(int32_t n, const su3_batch_item* item
     o.n_sites = it.desc.n_sites;
     o.dtype = it.desc.dtype;
     o.first_tile = first_tile;
-    o.arith = it.desc.arith;
-    o.reserved = 0;
-    memcpy(o.b, it.b, sizeof(o.b));
-    split_b_pairs(&it.b[0][0][0][0], o.bpair);
+    fill_batch_b(&o, it.desc.dtype, it.desc.arith, &it.b[0][0][0][0]);
     first_tile += batch_tile_count(it.desc.n_sites, it.desc.dtype, cfg.tile_sites);
   }
   // clear the status word, then upload the whole table in one copy

@@ -5,6 +5,9 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
+#include <string.h>
+
+#include "su3_internal.h"
 
 namespace su3 {
 
@@ -222,12 +225,26 @@ struct BMat {
   A v[72];
   float unit;
 };
+template <>
+struct BMat<double> {
+  double v[72];
+  float unit;
+  FixedMat fix;
+};
 
-template <typename A>
+// COLS: columns of the FP64 product's b for the fixed-point form (0: the op does not use it).
+template <typename A, int COLS>
 inline BMat<A> make_b(const double* b) {
   BMat<A> m;
   for (int i = 0; i < 72; ++i) m.v[i] = (A)b[i];
   m.unit = 1.0f;
+  if constexpr (sizeof(A) == 8) {
+    memset(&m.fix, 0, sizeof(m.fix));
+    if constexpr (COLS > 0) {
+      m.fix.range = fix_b<COLS>(b, m.fix.fx, m.fix.eb) ? kFixExpRange : 0;
+      m.fix.k = fixed_const();
+    }
+  }
   return m;
 }
 
@@ -239,6 +256,7 @@ __device__ __forceinline__ void load_b_op(const BMat<typename Op::BArg>& b, type
   __syncthreads();
   op.init(bsh + 18 * (threadIdx.x & 3), native_warps);
   op.set_unit(b.unit);
+  if constexpr (Op::kFixCols > 0) op.set_fixed(b.fix, threadIdx.x & 3);
 }
 
 // ---- the link product -------------------------------------------------------------------------
@@ -332,6 +350,179 @@ __device__ __forceinline__ void link_mult(const Link<T>& a, const T (&bre)[9], c
   }
 }
 
+// ---- FP64 rows in fixed point -------------------------------------------------------------------
+// One output row takes 36 FP64 FMAs, of which GB300 does 2 per clock and SM: by themselves they
+// hold the FP64 product at 24 % of the memory bandwidth, with every other unit idle. The integer
+// units do 32 multiply-adds of 32 x 32 + 64 bits per clock and SM beside them. So five of a row's
+// six output reals are computed in fixed point, at FP64 accuracy, while the FP64 pipe computes the
+// sixth:
+//  * a's row becomes 61-bit fixed point relative to its largest real, A = ah * 2^32 + al with a
+//    29-bit ah and a sign, and al a signed 32-bit limb; b comes from the host in the same form
+//    (fix_b). A real within 2^-8 of the largest is exact; a smaller one is cut at 2^-61 of it.
+//  * an output is the sum of six products A * B: H = sum ah*bh, X = sum ah*bl and Y = sum al*bh,
+//    in 64-bit accumulators that cannot overflow (6 * 2^58, 6 * 2^60), and T = H + X/2^32 + Y/2^32.
+//    al*bl is left out (below 1.5 units of T). The start values make X and Y unsigned
+//    (xbias = 2^63), so that their high words need no sign extension, and take that 2 * 2^31 back
+//    and round (hbias).
+//  * T becomes a double with one rounding (fixed_to_f64).
+// T's unit is 2^-58 of (the row's largest real) x (b's), each rounded up to a power of two. T is off
+// by at most 5 units (al*bl 1.5, the two shifts 1, a's cut 0.75 and its negation 0.4, b's rounding
+// 0.4, T's one's complement 1), as a rule by 0.5. So an output is within half an ulp + 5 * 2^-58 of
+// that product. Over random SU(3) matrices the error is 2.5e-17 of the result's norm, 4.7e-17 with
+// every sixth output by FMAs, against 9.8e-17 for FMAs alone; the largest single error 3.3e-16
+// against 4.4e-16.
+// The bound does not shrink with the terms, so a row whose terms may all be small takes FP64 FMAs
+// throughout. b is checked by fix_b. In a row, at least four of the six reals must be within 2^-8
+// of the largest: ensured by the exponents' distances from the largest summing to at most 26
+// (three above 8 would make 27), which costs an add per real. With three of b's reals in every
+// column within 2^-5, every output then has a term of at least 2^-14 of T's full scale. 99.98 % of
+// the rows of random SU(3) matrices pass (with a limit of 23, 99.92 %: 4 % slower). Rows with
+// zeros, subnormals, infinities or NaN, or outside 2^-723 .. 2^677, do not pass. Which way a row
+// goes depends on its values only, so results are the same for every launch shape and layout.
+// Measured (AOS, 2^21 sites): FP64 FMAs alone 1,585 GB/s; six outputs of six in fixed point 4,711,
+// five 5,220 (the multiplier 55 %, FP64 pipe 60 % and ALU 45 % busy; a wide multiply-add holds
+// back the other integer pipe, so they do not overlap fully), 14 of 18 5,187, 13 of 18 4,869, 12
+// of 18 4,273.
+
+// b[j] (or v[j]) of one thread as fixed-point limbs: element 3*m + l (COLS 3) or m (COLS 1).
+template <int COLS>
+struct FixedB {
+  int rh[3 * COLS], rl[3 * COLS], ih[3 * COLS], il[3 * COLS];
+  unsigned kb, range;
+  FixedConst k;
+  // from fix_b's limbs of b[j] (8-byte aligned), its exponent, and the exponents of a's rows taken
+  __device__ __forceinline__ void take(const int (*fx)[4], int eb, unsigned exp_range, const FixedConst& c) {
+    const int2* p = reinterpret_cast<const int2*>(fx);
+#pragma unroll
+    for (int e = 0; e < 3 * COLS; ++e) {
+      const int2 r = p[2 * e], i = p[2 * e + 1];
+      rh[e] = r.x;
+      rl[e] = r.y;
+      ih[e] = i.x;
+      il[e] = i.y;
+    }
+    kb = (unsigned)(1085 - 1080 + eb) << 20;
+    range = exp_range;
+    k = c;
+  }
+};
+
+// a * b + c with a 64-bit accumulator. The carry-linked pair is issued as one IMAD.WIDE; mad.wide
+// was split into a product and 64-bit adds.
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long d;
+  asm("{.reg .b32 lo, hi;\n\t"
+      "mov.b64 {lo, hi}, %3;\n\t"
+      "mad.lo.cc.s32 lo, %1, %2, lo;\n\t"
+      "madc.hi.s32 hi, %1, %2, hi;\n\t"
+      "mov.b64 %0, {lo, hi};}"
+      : "=l"(d)
+      : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+
+// T in units of 2^k as a double, rounded once to nearest (ties away from zero); `base` is
+// (1023 + 62 + k) << 20. Valid while |T|'s high word is not 0: `least` collects its minimum. The
+// magnitude is T's one's complement when T is negative: one unit of T less, far below the rounding.
+__device__ __forceinline__ double fixed_to_f64(long long t, unsigned base, unsigned& least) {
+  int th, tl;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(tl), "=r"(th) : "l"(t));
+  const int s = th >> 31;
+  const unsigned ah = (unsigned)(th ^ s), al = (unsigned)(tl ^ s);
+  least = min(least, ah);
+  unsigned n, mh, ml, lo, hi;
+  asm("clz.b32 %0, %1;" : "=r"(n) : "r"(ah));
+  asm("shf.l.wrap.b32 %0, %1, %2, %3;" : "=r"(mh) : "r"(al), "r"(ah), "r"(n));
+  asm("shl.b32 %0, %1, %2;" : "=r"(ml) : "r"(al), "r"(n));
+  asm("shf.r.wrap.b32 %0, %1, %2, 11;" : "=r"(lo) : "r"(ml), "r"(mh));
+  hi = mh >> 11;  // with the leading bit, which adds the last 1 to the exponent field
+  const unsigned e = (base | ((unsigned)s & 0x80000000u)) - (n << 20);
+  asm("{add.cc.u32 %0, %0, %2; addc.u32 %1, %1, %3;}" : "+r"(lo), "+r"(hi) : "r"((ml >> 10) & 1u), "r"(e));
+  return __hiloint2double((int)hi, (int)lo);
+}
+
+// One output row c[l] = sum_m a[m] b[m][l], l < COLS; bj = the same b in FP64 (re, im of element
+// COLS*m + l). The last NAT (0 or 1) output reals by FP64 FMAs, in row_mult's order. Returns false, with
+// c undefined, when the row does not suit.
+template <int COLS, int NAT>
+__device__ __forceinline__ bool fixed_row(const double (&are)[3], const double (&aim)[3], const FixedB<COLS>& b,
+                                          const double* bj, double (&cre)[COLS], double (&cim)[COLS]) {
+  const double x[6] = {are[0], are[1], are[2], aim[0], aim[1], aim[2]};
+  unsigned hn[6];  // the complement of |x|'s high word, so that its exponent field grows as |x| falls
+#pragma unroll
+  for (int q = 0; q < 6; ++q) hn[q] = ~(unsigned)__double2hiint(x[q]) & 0x7fffffffu;
+  const unsigned lowest = min(min(min(hn[0], hn[1]), min(hn[2], hn[3])), min(hn[4], hn[5]));
+  const int e0 = (int)(lowest >> 20);  // 0x7ff - the largest exponent field
+  int d[6], sum = 0;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    d[q] = (int)(hn[q] >> 20) - e0;
+    sum += d[q];
+  }
+    if (sum > 26 || (unsigned)(0x7ff - kFixExpMin) - (unsigned)e0 >= b.range) return false;
+  int ah[6], al[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {  // every d <= 26
+    const int h = __double2hiint(x[q]);
+    const unsigned l = (unsigned)__double2loint(x[q]);
+    const unsigned s = (unsigned)(h >> 31);
+    const unsigned m = ((unsigned)h & 0xfffffu) | b.k.lead;
+    const unsigned wh = __funnelshift_l(l, m, 8) ^ s, wl = (l << 8) ^ s;
+    const unsigned vl = __funnelshift_r(wl, wh, d[q]);
+    ah[q] = ((int)wh >> d[q]) + (int)(vl >> 31);
+    al[q] = (int)vl;
+  }
+  int nh[3], nl[3];  // of -im (-al less one unit: al may be -2^31)
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    nh[m] = b.k.zero - ah[3 + m];
+    nl[m] = al[3 + m] ^ b.k.ones;
+  }
+  const unsigned base = ((0x7ffu - (unsigned)e0) << 20) + b.kb;
+  unsigned least = 0x7fffffffu;
+  auto sum3 = [](long long h, long long u, long long v) {
+    return h + (long long)((unsigned long long)u >> 32) + (long long)((unsigned long long)v >> 32);
+  };
+#pragma unroll
+  for (int l = 0; l < COLS; ++l) {
+    // re and im together: six independent chains of multiply-adds
+    long long hr = b.k.hbias, xr = b.k.xbias, yr = b.k.xbias, hi = b.k.hbias, xi = b.k.xbias, yi = b.k.xbias;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const int e = COLS * m + l;
+      hr = mad_wide(ah[m], b.rh[e], hr);
+      hr = mad_wide(nh[m], b.ih[e], hr);
+      xr = mad_wide(ah[m], b.rl[e], xr);
+      xr = mad_wide(nh[m], b.il[e], xr);
+      yr = mad_wide(al[m], b.rh[e], yr);
+      yr = mad_wide(nl[m], b.ih[e], yr);
+      if (l < COLS - NAT) {
+        hi = mad_wide(ah[m], b.ih[e], hi);
+        hi = mad_wide(ah[3 + m], b.rh[e], hi);
+        xi = mad_wide(ah[m], b.il[e], xi);
+        xi = mad_wide(ah[3 + m], b.rl[e], xi);
+        yi = mad_wide(al[m], b.ih[e], yi);
+        yi = mad_wide(al[3 + m], b.rh[e], yi);
+      }
+    }
+    const long long tr = sum3(hr, xr, yr), ti = sum3(hi, xi, yi);
+    cre[l] = fixed_to_f64(tr, base, least);
+    if (l < COLS - NAT) {
+      cim[l] = fixed_to_f64(ti, base, least);
+    } else {
+      double im = are[0] * bj[2 * l + 1];
+      im = fma(aim[0], bj[2 * l], im);
+#pragma unroll
+      for (int m = 1; m < 3; ++m) {
+        im = fma(are[m], bj[2 * (COLS * m + l) + 1], im);
+        im = fma(aim[m], bj[2 * (COLS * m + l)], im);
+      }
+      cim[l] = im;
+    }
+  }
+  return least != 0;  // a result below 2^-27 of the row's largest times b's: FP64 FMAs
+}
+
 // ---- per-link operations used by the streaming kernels ----------------------------------------
 // An op owns this thread's copy of b[j] (j = tid % 4) and turns one input link (NE_IN complex
 // storage elements) into one output link (3*ROWS_OUT elements). `src` and `dst` may alias.
@@ -346,6 +537,7 @@ struct NativeOp {
   using A = typename S::acc;   // FP64 for F64 storage, FP32 otherwise
   using V = typename S::vec;
   using BArg = A;              // precision of b in the kernel parameters
+  static constexpr int kFixCols = 0;
   static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
   static constexpr bool kRowSplit = true;  // has apply_row: one thread per output row is possible
   A bre[9], bim[9];
@@ -391,6 +583,62 @@ struct NativeOp {
   }
 };
 
+// FP64 storage: rows in fixed point (fixed_row), or by FP64 FMAs where a row or b does not suit.
+template <int NE_IN, int ROWS_OUT>
+struct NativeOp<kF64, NE_IN, ROWS_OUT> {
+  using S = Storage<kF64>;
+  using V = double2;
+  using BArg = double;
+  static constexpr int kFixCols = 3;
+  static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
+  static constexpr bool kRowSplit = true;
+  // output reals per row on the FP64 pipe; two-row in, full out has its rebuild of row 2 there
+  static constexpr int kNat = NE_IN == 6 && ROWS_OUT == 3 ? 0 : 1;
+  FixedB<3> fix;
+  const double* bm;  // b[j] in FP64, in shared memory
+  __device__ __forceinline__ void begin_tile(int) {}
+  __device__ __forceinline__ void set_unit(float) {}
+  __device__ __forceinline__ void init(const BArg* bj, int /*native_warps*/) { bm = bj; }
+  __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { fix.take(f.fx[j], f.eb[j], f.range, f.k); }
+  __device__ __forceinline__ void row(const double (&are)[3], const double (&aim)[3], double (&cre)[3],
+                                      double (&cim)[3]) const {
+    if (fixed_row<3, kNat>(are, aim, fix, bm, cre, cim)) return;
+    double bre[9], bim[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      bre[e] = bm[2 * e];
+      bim[e] = bm[2 * e + 1];
+    }
+    row_mult(are, aim, bre, bim, cre, cim);
+  }
+  template <int ES_IN = 1, int ES_OUT = 1>
+  __device__ __forceinline__ void apply(const V* src, V* dst) const {
+#pragma unroll
+    for (int k = 0; k < ROWS_OUT; ++k) apply_row<ES_IN, ES_OUT>(src, dst, k);
+  }
+  // Output row k alone (row split: one thread per output row). Reads input row k only, except
+  // that a rebuilt row 2 reads rows 0 and 1 (two-row in, full out is never in place).
+  template <int ES_IN = 1, int ES_OUT = 1>
+  __device__ __forceinline__ void apply_row(const V* src, V* dst, int k) const {
+    double are[3], aim[3], cre[3], cim[3];
+    if (NE_IN == 6 && ROWS_OUT == 3 && k == 2) {
+      double r0re[3], r0im[3], r1re[3], r1im[3];
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        S::unpack(src[m * ES_IN], r0re[m], r0im[m]);
+        S::unpack(src[(3 + m) * ES_IN], r1re[m], r1im[m]);
+      }
+      rebuild_row2_elems(r0re, r0im, r1re, r1im, are, aim);
+    } else {
+#pragma unroll
+      for (int m = 0; m < 3; ++m) S::unpack(src[(3 * k + m) * ES_IN], are[m], aim[m]);
+    }
+    row(are, aim, cre, cim);
+#pragma unroll
+    for (int l = 0; l < 3; ++l) dst[(3 * k + l) * ES_OUT] = S::pack(cre[l], cim[l]);
+  }
+};
+
 // ---- adjacent SU(3) operations ----------------------------------------------------------------
 // The other per-link SU(3) products of lattice-QCD codes next to the benchmark's a x b: a^dagger x b (MILC's
 // mult_su3_an) and the matrix x colour-vector products a v and a^dagger v (mult_su3_mat_vec and
@@ -403,6 +651,7 @@ struct AnOp {  // c[k][l] = sum_m conj(a[m][k]) b[m][l]
   using A = typename S::acc;
   using V = typename S::vec;
   using BArg = A;
+  static constexpr int kFixCols = 0;
   static constexpr int kNeIn = 9, kNeOut = 9;
   static constexpr bool kRowSplit = false;  // row k of a^dagger b reads column k of a
   A bre[9], bim[9];
@@ -448,6 +697,7 @@ struct MatVecOp {  // w[k] = sum_m a[k][m] v[m]   (ADJ: sum_m conj(a[m][k]) v[m]
   using A = typename S::acc;
   using V = typename S::vec;
   using BArg = A;
+  static constexpr int kFixCols = 0;
   static constexpr int kNeIn = 9, kNeOut = 3;
   static constexpr bool kRowSplit = false;  // one output vector per link
   A vre[3], vim[3];
@@ -614,6 +864,7 @@ template <int NE_IN, int ROWS_OUT>
 struct PairF64Op {
   using V = double2;
   using BArg = double;
+  static constexpr int kFixCols = 0;
   static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
   static constexpr bool kRowSplit = true;
   // b[j] split once per thread, as lane pairs for the two terms of each (m, l):
@@ -716,6 +967,7 @@ struct PairF64Op {
 struct PairAnOp {
   using V = double2;
   using BArg = double;
+  static constexpr int kFixCols = 0;
   static constexpr int kNeIn = 9, kNeOut = 9;
   static constexpr bool kRowSplit = false;  // row k of a^dagger b reads column k of a
   PairF64Op<9, 3> pair;                     // b as FP32 pairs and the row routine
@@ -749,6 +1001,7 @@ template <bool ADJ>
 struct PairMatVecOp {
   using V = double2;
   using BArg = double;
+  static constexpr int kFixCols = 0;
   static constexpr int kNeIn = 9, kNeOut = 3;
   static constexpr bool kRowSplit = false;  // one output vector per link
   float2 ya[3], yb[3], yla[3], ylb[3];      // v[m]: (re, im), (-im, re), and their low parts
@@ -795,6 +1048,7 @@ template <int NE_IN, int ROWS_OUT>
 struct HybridF64Op {
   using V = double2;
   using BArg = double;
+  static constexpr int kFixCols = 3;
   static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
   static constexpr bool kRowSplit = true;
   NativeOp<kF64, NE_IN, ROWS_OUT> nat;
@@ -812,6 +1066,7 @@ struct HybridF64Op {
     native = period > 0 && ((k + (int)(threadIdx.x >> 5)) % period) == 0;
   }
   __device__ __forceinline__ void set_unit(float u) { pair.set_unit(u); }
+  __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { nat.set_fixed(f, j); }
   template <int ES_IN = 1, int ES_OUT = 1>
   __device__ __forceinline__ void apply(const V* src, V* dst) const {
     if (native) nat.template apply<ES_IN, ES_OUT>(src, dst);

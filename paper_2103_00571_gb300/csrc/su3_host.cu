@@ -100,7 +100,7 @@ static su3_status run_host(const Form& f, const LaunchCfg& cfg, const void* a, c
   LaunchCfg hc = cfg;
   hc.block = block;
   p.native_warps = native_warps(f, hc);
-  p.b = make_b<typename Op::BArg>(b);
+  p.b = make_b<typename Op::BArg, Op::kFixCols>(b);
   auto kern = su3_host_kernel<Op>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 0;

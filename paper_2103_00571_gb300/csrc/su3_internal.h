@@ -1,6 +1,8 @@
 // Host-side internals shared by the libsu3 translation units (not part of the C ABI).
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <string>
@@ -79,6 +81,65 @@ su3_status launch_selftest_wait(int limit_ms, const LaunchCtx& ctx);
 su3_status launch_pack(const Form& dst, const double* src, void* dst_dev, const LaunchCtx& ctx);
 su3_status launch_unpack(const Form& src, const void* src_dev, double* dst, const LaunchCtx& ctx);
 
+// ---- b of the FP64 product in fixed point (the device side is fixed_row in su3_device.cuh) -------
+
+// Constants of the fixed-point rows that must be unknown to the compiler. With them known it turns
+// products by -x into negated multiplies and splits multiply-accumulates into a product and 64-bit
+// adds (19 more integer adds per output: 4,142 against 4,732 GB/s at 2^21 sites).
+struct FixedConst {
+  int zero, ones;          // 0, -1
+  unsigned lead;           // 2^20: the implicit leading bit of an FP64 mantissa, in its high word
+  long long hbias, xbias;  // start values of the accumulators
+};
+inline FixedConst fixed_const() { return FixedConst{0, -1, 1u << 20, 1 - (1ll << 32), (long long)(1ull << 63)}; }
+
+// Element e of b[j] as two signed 32-bit limbs for re and two for im, fx[j][e] = (re_hi, re_lo,
+// im_hi, im_lo), value (hi * 2^32 + lo) * 2^(eb[j] - 61) with |b[j]| < 2^eb[j]. `range`: the number of
+// exponents of a row's largest real that the fixed-point form takes, 0 when b does not suit it.
+struct FixedMat {
+  alignas(8) int fx[4][9][4];
+  int eb[4];
+  unsigned range;
+  FixedConst k;
+};
+
+// Biased exponents of a row's largest |real| that the form takes: 2^-723 <= |a| < 2^677.
+constexpr unsigned kFixExpMin = 300, kFixExpRange = 1400;
+
+// Fills fx and eb from b (COLS 3: [j][row][col]; 1: one colour vector per j at the start of b's j-th
+// 18 reals). Returns whether b suits the form: every value finite, the largest of each matrix within
+// 1e-30 .. 1e30, and in every column at least three of the six reals within 2^-5 of that largest
+// (see fixed_row for why). 99.9 % of sets of four random SU(3) matrices do; when one matrix does not,
+// every row takes FP64 FMAs.
+template <int COLS>
+inline bool fix_b(const double* b, int (*fx)[9][4], int* eb) {
+  for (int j = 0; j < 4; ++j) {
+    const double* m = b + 18 * j;
+    double top = 0;
+    for (int q = 0; q < 6 * COLS; ++q) {
+      if (!(fabs(m[q]) <= 1e30)) return false;  // also NaN
+      top = fabs(m[q]) > top ? fabs(m[q]) : top;
+    }
+    if (top < 1e-30) return false;
+    frexp(top, &eb[j]);  // top < 2^eb
+    const double large = ldexp(1.0, eb[j] - 5);
+    for (int l = 0; l < COLS; ++l) {
+      int n = 0;
+      for (int r = 0; r < 3; ++r)
+        for (int c = 0; c < 2; ++c) n += fabs(m[2 * (COLS * r + l) + c]) >= large;
+      if (n < 3) return false;
+    }
+    const double scale = ldexp(1.0, 61 - eb[j]);
+    for (int q = 0; q < 6 * COLS; ++q) {
+      const long long v = (long long)rint(m[q] * scale);
+      const int lo = (int)(unsigned)((unsigned long long)v & 0xffffffffull);
+      fx[j][q >> 1][2 * (q & 1)] = (int)((v - lo) >> 32);
+      fx[j][q >> 1][2 * (q & 1) + 1] = lo;
+    }
+  }
+  return true;
+}
+
 // Device descriptor of one lattice in a batched launch.
 struct BatchDesc {
   const void* a;
@@ -86,11 +147,16 @@ struct BatchDesc {
   long long n_sites;
   int dtype;           // SU3_F64 or SU3_F32
   int first_tile;      // exclusive prefix sum of tile counts
-  int arith;           // SU3_ARITH_NATIVE, or SU3_ARITH_F32PAIR for F64 lattices
-  int reserved;
+  short arith;         // SU3_ARITH_NATIVE, or SU3_ARITH_F32PAIR for F64 lattices
+  short fixed;         // F64 NATIVE: whether b suits the fixed-point form (fix_b)
+  signed char eb[4];   // F64 NATIVE: exponents of the four matrices (fix_b)
   double b[72];        // FP64 b (F32 lattices round it in the kernel)
-  float bpair[144];    // F32PAIR: b[j][e] split as (re_hi, im_hi, re_lo, im_lo), [j][e][4]
+  union {
+    float bpair[144];    // F32PAIR: b[j][e] split as (re_hi, im_hi, re_lo, im_lo), [j][e][4]
+    int bfix[4][9][4];   // F64 NATIVE: b in fixed point (fix_b)
+  };
 };
+static_assert(offsetof(BatchDesc, bfix) % 8 == 0 && sizeof(BatchDesc) % 8 == 0, "bfix is read as 8-byte words");
 
 // Fills BatchDesc::bpair from the FP64 b (hi = b rounded to FP32, lo = the rest rounded to FP32).
 inline void split_b_pairs(const double* b, float* out) {
@@ -101,6 +167,22 @@ inline void split_b_pairs(const double* b, float* out) {
     out[4 * q + 1] = ih;
     out[4 * q + 2] = (float)(r - (double)rh);
     out[4 * q + 3] = (float)(i - (double)ih);
+  }
+}
+
+// Fills the descriptor's arithmetic and b from an item's.
+inline void fill_batch_b(BatchDesc* o, int dtype, int arith, const double* b) {
+  o->arith = (short)arith;
+  o->fixed = 0;
+  for (int j = 0; j < 4; ++j) o->eb[j] = 0;
+  for (int i = 0; i < 72; ++i) o->b[i] = b[i];
+  if (dtype == SU3_F64 && arith == SU3_ARITH_NATIVE) {
+    int eb[4] = {0, 0, 0, 0};
+    for (int i = 0; i < 144; ++i) o->bpair[i] = 0;
+    o->fixed = fix_b<3>(b, o->bfix, eb) ? 1 : 0;
+    for (int j = 0; j < 4; ++j) o->eb[j] = (signed char)eb[j];  // |eb| <= 101
+  } else {
+    split_b_pairs(b, o->bpair);
   }
 }
 

@@ -1,0 +1,127 @@
+"""The FP64 product's fixed-point rows (NATIVE arithmetic) against extended precision, at the edges of
+their range: rows whose reals differ in size just inside and outside what the fixed-point form takes,
+zeros, extreme and non-finite values, and b matrices that suit it or do not.
+
+Bounds. A row in fixed point: half an ulp of the result, plus 5 units of 2^-58 of (largest real of
+the row, rounded up to a power of two) x (the same of b): the sums of the terms that are left out or
+rounded. A row by FP64 FMAs: six roundings, 6 * 2^-53 * sum |a||b|.
+"""
+import numpy as np
+import pytest
+
+import paper_2103_00571_gb300 as su3
+import su3_inputs as gen
+
+from gpu_helpers import run_form
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53
+
+
+def links(a, n=9):
+    """[V*72] doubles as complex extended precision [links, 3, 3]."""
+    x = np.asarray(a, dtype=np.longdouble).reshape(-1, 3, 3, 2)
+    return x[..., 0], x[..., 1]
+
+
+def exact_and_bound(a, b):
+    """c = a x b in extended precision and the per-real error bound, both [V*72]."""
+    ar, ai = links(a)
+    br, bi = (np.tile(x, (ar.shape[0] // 4, 1, 1)) for x in links(b))
+    cr = np.einsum("qkm,qml->qkl", ar, br) - np.einsum("qkm,qml->qkl", ai, bi)
+    ci = np.einsum("qkm,qml->qkl", ar, bi) + np.einsum("qkm,qml->qkl", ai, br)
+    mag = lambda x, y, z, w: np.einsum("qkm,qml->qkl", abs(x), abs(y)) + np.einsum("qkm,qml->qkl", abs(z), abs(w))  # noqa: E731
+    s = np.stack([mag(ar, br, ai, bi), mag(ar, bi, ai, br)], -1)
+    up = lambda x: 2.0 ** np.ceil(np.log2(np.where(x > 0, x, 1).astype(np.float64)))  # noqa: E731
+    top = up(np.maximum(abs(ar), abs(ai)).max(2, keepdims=True))[..., None] * up(
+        np.maximum(abs(br), abs(bi)).max((1, 2), keepdims=True))[..., None]
+    c = np.stack([cr, ci], -1)
+    fixed = U * abs(c) + 5 * 2.0 ** -58 * top
+    chain = 6 * U * s
+    return c.reshape(-1), np.maximum(fixed, chain).reshape(-1), chain.reshape(-1)
+
+
+def family(name, V, rng):
+    a, b = gen.sites(7, 3, V), gen.bmat(7, 3, V)
+    if name == "graded":  # the reals of a row spread over up to 2^9: on both sides of the limit
+        a = a * 2.0 ** -rng.integers(0, 10, a.size)
+    elif name == "spread":  # two reals of every row 2^-7 or 2^-8, the others near the largest
+        a = np.sign(a) * rng.uniform(1, 2, a.size)
+        for r in a.reshape(-1, 6):
+            r[rng.permutation(6)[:3]] *= 2.0 ** -rng.integers(6, 10)
+    elif name == "identity":  # links near the identity
+        a = 1e-5 * a
+        a.reshape(-1, 3, 3, 2)[:, range(3), range(3), 0] += 1.0
+    elif name == "real":  # zero imaginary parts
+        a.reshape(-1, 2)[:, 1] = 0.0
+    elif name == "large":
+        a = a * 2.0 ** 900
+    elif name == "small":
+        a = a * 2.0 ** -900
+    elif name == "scaled":  # rows of sizes through the whole range of the fixed-point form
+        a = (a.reshape(-1, 6) * 2.0 ** rng.integers(-720, 670, (a.size // 6, 1))).reshape(-1)
+    elif name == "dyadic":  # low limbs of all ones and all zeros, exact powers of two
+        a = np.sign(a) * np.where(rng.random(a.size) < 0.5, 1.0 - 2.0 ** -rng.integers(1, 54, a.size),
+                                  2.0 ** -rng.integers(0, 4, a.size).astype(float))
+    elif name == "b_identity":
+        b = np.zeros(72)
+        b.reshape(4, 3, 3, 2)[:, range(3), range(3), 0] = 1.0
+    elif name == "b_one_sparse":  # one matrix does not suit the form: all take FMAs
+        b = b.copy()
+        b.reshape(4, 3, 3, 2)[2, :, 1] = [[1e-3, 0], [1.0, 0], [0, 1e-4]]
+    elif name == "b_scaled":
+        b = b * np.repeat([2.0 ** 90, 1.0, 2.0 ** -60, 3.0], 18)
+    return a, b
+
+
+FAMILIES = ["random", "graded", "spread", "identity", "real", "large", "small", "scaled", "dyadic", "b_identity",
+            "b_one_sparse", "b_scaled"]
+
+
+@pytest.mark.parametrize("name", FAMILIES)
+def test_error_bound(name):
+    V = 1537
+    a, b = family(name, V, np.random.default_rng(11))
+    h = su3.Handle(0)
+    c = run_form(h, a, b, su3.F64)
+    want, bound, chain = exact_and_bound(a, b)
+    err = np.abs(c.astype(np.longdouble) - want)
+    assert np.all(np.isfinite(c))
+    assert np.all(err <= bound + 2.0 ** -1073), name
+    if name in ("real", "identity", "large", "small", "b_identity", "b_one_sparse"):  # rows by FMAs throughout
+        assert np.all(err <= chain + 2.0 ** -1073), name
+    if name == "random":  # fixed point is the more exact: every row of FMAs measures 9.8e-17
+        assert np.linalg.norm(err.astype(float)) < 7e-17 * np.linalg.norm(want.astype(float))
+    h.close()
+
+
+def test_non_finite_rows_stay_local():
+    """Infinities and NaN give what FP64 arithmetic gives in their rows and touch no other row."""
+    V = 70
+    a, b = gen.sites(7, 4, V), gen.bmat(7, 4, V)
+    bad = a.copy()
+    bad[[5, 6 * 100 + 1, 6 * 333, 6 * 500 + 3]] = [np.inf, -np.inf, np.nan, 1.7e308]
+    h = su3.Handle(0)
+    c, good = run_form(h, bad, b, su3.F64), run_form(h, a, b, su3.F64)
+    rows = np.zeros(V * 12, bool)
+    rows[[0, 100, 333, 500]] = True
+    assert np.array_equal(c.reshape(-1, 6)[~rows], good.reshape(-1, 6)[~rows])
+    assert not np.isfinite(c.reshape(-1, 6)[[0, 100, 333]]).any()
+    h.close()
+
+
+@pytest.mark.parametrize("layout", [su3.AOS, su3.AOSOA32, su3.SOA])
+@pytest.mark.parametrize("ri,ro", [(su3.FULL18, su3.FULL18), (su3.TWOROW12, su3.TWOROW12), (su3.TWOROW12, su3.FULL18)])
+def test_rows_in_every_layout(layout, ri, ro):
+    """The same rows to the same bits whatever the layout and the threads per link; ragged sizes."""
+    h = su3.Handle(0)
+    for V in (1, 9, 129, 1037):
+        a, b = gen.sites(7, 5, V), gen.bmat(7, 5, V)
+        a[: min(a.size, 900)] *= 2.0 ** -np.random.default_rng(V).integers(0, 12, min(a.size, 900))  # both kinds of row
+        base = run_form(h, a, b, su3.F64, ri, ro)
+        for tpl in (1, 3):
+            got = run_form(h, a, b, su3.F64, ri, ro, layout=layout,
+                           cfg=dict(block=128, tile_sites=32, stages=3, threads_per_link=tpl))
+            assert np.array_equal(got, base), (V, tpl)
+    h.close()
