@@ -441,35 +441,47 @@ __device__ __forceinline__ double fixed_to_f64(long long t, unsigned base, unsig
   return __hiloint2double((int)hi, (int)lo);
 }
 
-// One output row c[l] = sum_m a[m] b[m][l], l < COLS; bj = the same b in FP64 (re, im of element
-// COLS*m + l). The last NAT (0 or 1) output reals by FP64 FMAs, in row_mult's order. Returns false, with
-// c undefined, when the row does not suit.
-template <int COLS, int NAT>
-__device__ __forceinline__ bool fixed_row(const double (&are)[3], const double (&aim)[3], const FixedB<COLS>& b,
-                                          const double* bj, double (&cre)[COLS], double (&cim)[COLS]) {
-  const double x[6] = {are[0], are[1], are[2], aim[0], aim[1], aim[2]};
-  unsigned hn[6];  // the complement of |x|'s high word, so that its exponent field grows as |x| falls
+// Whether a row (reals a[0..2].re, a[0..2].im) suits the fixed-point form: the distances d of its
+// exponents from the largest, each at most 26, and e0 = 0x7ff - the largest exponent field.
+struct FixedExps {
+  int d[6], e0;
+  __device__ __forceinline__ bool take(const double (&are)[3], const double (&aim)[3], unsigned range) {
+    unsigned hn[6];  // the complement of |x|'s high word, so that its exponent field grows as |x| falls
 #pragma unroll
-  for (int q = 0; q < 6; ++q) hn[q] = ~(unsigned)__double2hiint(x[q]) & 0x7fffffffu;
-  const unsigned lowest = min(min(min(hn[0], hn[1]), min(hn[2], hn[3])), min(hn[4], hn[5]));
-  const int e0 = (int)(lowest >> 20);  // 0x7ff - the largest exponent field
-  int d[6], sum = 0;
+    for (int m = 0; m < 3; ++m) {
+      hn[m] = ~(unsigned)__double2hiint(are[m]) & 0x7fffffffu;
+      hn[3 + m] = ~(unsigned)__double2hiint(aim[m]) & 0x7fffffffu;
+    }
+    const unsigned lowest = min(min(min(hn[0], hn[1]), min(hn[2], hn[3])), min(hn[4], hn[5]));
+    e0 = (int)(lowest >> 20);
+    int sum = 0;
 #pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    d[q] = (int)(hn[q] >> 20) - e0;
-    sum += d[q];
+    for (int q = 0; q < 6; ++q) {
+      d[q] = (int)(hn[q] >> 20) - e0;
+      sum += d[q];
+    }
+    return sum <= 26 && (unsigned)(0x7ff - kFixExpMin) - (unsigned)e0 < range;
   }
-    if (sum > 26 || (unsigned)(0x7ff - kFixExpMin) - (unsigned)e0 >= b.range) return false;
+};
+
+// One output row c[l] = sum_m a[m] b[m][l], l < COLS, of a row whose exponents suit; bj = the same b
+// in FP64 (re, im of element COLS*m + l). The last NAT (0 or 1) output reals by FP64 FMAs, in
+// row_mult's order. Returns false, with c undefined, when a result is too small for the form.
+template <int COLS, int NAT>
+__device__ __forceinline__ bool fixed_row(const double (&are)[3], const double (&aim)[3], const FixedExps& ex,
+                                          const FixedB<COLS>& b, const double* bj, double (&cre)[COLS],
+                                          double (&cim)[COLS]) {
+  const double x[6] = {are[0], are[1], are[2], aim[0], aim[1], aim[2]};
   int ah[6], al[6];
 #pragma unroll
-  for (int q = 0; q < 6; ++q) {  // every d <= 26
+  for (int q = 0; q < 6; ++q) {
     const int h = __double2hiint(x[q]);
     const unsigned l = (unsigned)__double2loint(x[q]);
     const unsigned s = (unsigned)(h >> 31);
     const unsigned m = ((unsigned)h & 0xfffffu) | b.k.lead;
     const unsigned wh = __funnelshift_l(l, m, 8) ^ s, wl = (l << 8) ^ s;
-    const unsigned vl = __funnelshift_r(wl, wh, d[q]);
-    ah[q] = ((int)wh >> d[q]) + (int)(vl >> 31);
+    const unsigned vl = __funnelshift_r(wl, wh, ex.d[q]);
+    ah[q] = ((int)wh >> ex.d[q]) + (int)(vl >> 31);
     al[q] = (int)vl;
   }
   int nh[3], nl[3];  // of -im (-al less one unit: al may be -2^31)
@@ -478,7 +490,7 @@ __device__ __forceinline__ bool fixed_row(const double (&are)[3], const double (
     nh[m] = b.k.zero - ah[3 + m];
     nl[m] = al[3 + m] ^ b.k.ones;
   }
-  const unsigned base = ((0x7ffu - (unsigned)e0) << 20) + b.kb;
+  const unsigned base = ((0x7ffu - (unsigned)ex.e0) << 20) + b.kb;
   unsigned least = 0x7fffffffu;
   auto sum3 = [](long long h, long long u, long long v) {
     return h + (long long)((unsigned long long)u >> 32) + (long long)((unsigned long long)v >> 32);
@@ -537,7 +549,7 @@ struct NativeOp {
   using A = typename S::acc;   // FP64 for F64 storage, FP32 otherwise
   using V = typename S::vec;
   using BArg = A;              // precision of b in the kernel parameters
-  static constexpr int kFixCols = 0;
+  static constexpr int kFixCols = 0, kMinCtas = 0;
   static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
   static constexpr bool kRowSplit = true;  // has apply_row: one thread per output row is possible
   A bre[9], bim[9];
@@ -590,6 +602,7 @@ struct NativeOp<kF64, NE_IN, ROWS_OUT> {
   using V = double2;
   using BArg = double;
   static constexpr int kFixCols = 3;
+  static constexpr int kMinCtas = 1;
   static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
   static constexpr bool kRowSplit = true;
   // output reals per row on the FP64 pipe; two-row in, full out has its rebuild of row 2 there
@@ -602,7 +615,8 @@ struct NativeOp<kF64, NE_IN, ROWS_OUT> {
   __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { fix.take(f.fx[j], f.eb[j], f.range, f.k); }
   __device__ __forceinline__ void row(const double (&are)[3], const double (&aim)[3], double (&cre)[3],
                                       double (&cim)[3]) const {
-    if (fixed_row<3, kNat>(are, aim, fix, bm, cre, cim)) return;
+    FixedExps ex;
+    if (ex.take(are, aim, fix.range) && fixed_row<3, kNat>(are, aim, ex, fix, bm, cre, cim)) return;
     double bre[9], bim[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
@@ -613,6 +627,29 @@ struct NativeOp<kF64, NE_IN, ROWS_OUT> {
   }
   template <int ES_IN = 1, int ES_OUT = 1>
   __device__ __forceinline__ void apply(const V* src, V* dst) const {
+    if constexpr (NE_IN == 6 && ROWS_OUT == 3) {
+      // two-row in, full out (never in place): row 2 is rebuilt first, so that the FP64 pipe works on
+      // it beside rows 0 and 1 (2,886 against 2,825 GB/s at L=48; the same operations as apply_row, so
+      // the same bits)
+      double r0re[3], r0im[3], r1re[3], r1im[3], r2re[3], r2im[3], cre[3], cim[3];
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        S::unpack(src[m * ES_IN], r0re[m], r0im[m]);
+        S::unpack(src[(3 + m) * ES_IN], r1re[m], r1im[m]);
+      }
+      rebuild_row2_elems(r0re, r0im, r1re, r1im, r2re, r2im);
+      auto put = [&](int k) {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) dst[(3 * k + l) * ES_OUT] = S::pack(cre[l], cim[l]);
+      };
+      row(r0re, r0im, cre, cim);
+      put(0);
+      row(r1re, r1im, cre, cim);
+      put(1);
+      row(r2re, r2im, cre, cim);
+      put(2);
+      return;
+    }
 #pragma unroll
     for (int k = 0; k < ROWS_OUT; ++k) apply_row<ES_IN, ES_OUT>(src, dst, k);
   }
@@ -651,7 +688,7 @@ struct AnOp {  // c[k][l] = sum_m conj(a[m][k]) b[m][l]
   using A = typename S::acc;
   using V = typename S::vec;
   using BArg = A;
-  static constexpr int kFixCols = 0;
+  static constexpr int kFixCols = 0, kMinCtas = 0;
   static constexpr int kNeIn = 9, kNeOut = 9;
   static constexpr bool kRowSplit = false;  // row k of a^dagger b reads column k of a
   A bre[9], bim[9];
@@ -697,7 +734,7 @@ struct MatVecOp {  // w[k] = sum_m a[k][m] v[m]   (ADJ: sum_m conj(a[m][k]) v[m]
   using A = typename S::acc;
   using V = typename S::vec;
   using BArg = A;
-  static constexpr int kFixCols = 0;
+  static constexpr int kFixCols = 0, kMinCtas = 0;
   static constexpr int kNeIn = 9, kNeOut = 3;
   static constexpr bool kRowSplit = false;  // one output vector per link
   A vre[3], vim[3];
@@ -729,6 +766,88 @@ struct MatVecOp {  // w[k] = sum_m a[k][m] v[m]   (ADJ: sum_m conj(a[m][k]) v[m]
       }
       dst[k * ES_OUT] = S::pack(re, im);
     }
+  }
+};
+
+// The same for FP64 storage, rows in fixed point (fixed_row): row k of a^dagger b is the conjugate of
+// a's column k times b, and an element of a v is a's row k times the one column v (all in fixed point:
+// with one of six on the FP64 pipe a^dagger v measured 9 % slower). At L=48, FP64 FMAs before:
+// a^dagger b 1,568 -> 4,590 GB/s, a v 2,960 -> 6,139, a^dagger v 2,950 -> 5,648 (the products' launch shape).
+template <>
+struct AnOp<kF64> {
+  using V = double2;
+  using BArg = double;
+  static constexpr int kFixCols = 3;
+  static constexpr int kMinCtas = 2;  // 128 registers: 148 otherwise, which the product's 4 x 128 threads exceed
+  static constexpr int kNeIn = 9, kNeOut = 9;
+  static constexpr bool kRowSplit = false;  // row k of a^dagger b reads column k of a
+  NativeOp<kF64, 9, 3> op;                  // b and the row routine
+  __device__ __forceinline__ void begin_tile(int) {}
+  __device__ __forceinline__ void set_unit(float) {}
+  __device__ __forceinline__ void init(const BArg* bj, int w) { op.init(bj, w); }
+  __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { op.set_fixed(f, j); }
+  template <int ES_IN = 1, int ES_OUT = 1>
+  __device__ __forceinline__ void apply(const V* src, V* dst) const {
+    double2 a[9];  // all of a first: the output may overwrite it (in place)
+#pragma unroll
+    for (int e = 0; e < 9; ++e) a[e] = src[e * ES_IN];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      double are[3], aim[3], cre[3], cim[3];
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        are[m] = a[3 * m + k].x;
+        aim[m] = -a[3 * m + k].y;
+      }
+      op.row(are, aim, cre, cim);
+#pragma unroll
+      for (int l = 0; l < 3; ++l) dst[(3 * k + l) * ES_OUT] = make_double2(cre[l], cim[l]);
+    }
+  }
+};
+
+template <bool ADJ>
+struct MatVecOp<kF64, ADJ> {
+  using V = double2;
+  using BArg = double;
+  static constexpr int kFixCols = 1;
+  static constexpr int kMinCtas = 1;
+  static constexpr int kNeIn = 9, kNeOut = 3;
+  static constexpr bool kRowSplit = false;  // one output vector per link
+  FixedB<1> fix;
+  const double* vm;  // v[j] in FP64, in shared memory
+  __device__ __forceinline__ void begin_tile(int) {}
+  __device__ __forceinline__ void set_unit(float) {}
+  __device__ __forceinline__ void init(const BArg* vj, int) { vm = vj; }
+  __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { fix.take(f.fx[j], f.eb[j], f.range, f.k); }
+  template <int ES_IN, int ES_OUT>
+  __device__ __forceinline__ void element(const V* src, V* dst, int k) const {
+    double are[3], aim[3], wre[1], wim[1];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const double2 x = src[(ADJ ? 3 * m + k : 3 * k + m) * ES_IN];
+      are[m] = x.x;
+      aim[m] = ADJ ? -x.y : x.y;
+    }
+    FixedExps ex;
+    if (!(ex.take(are, aim, fix.range) && fixed_row<1, 0>(are, aim, ex, fix, vm, wre, wim))) {
+      double re = 0, im = 0;
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        re = fma(are[m], vm[2 * m], re);
+        re = fma(-aim[m], vm[2 * m + 1], re);
+        im = fma(are[m], vm[2 * m + 1], im);
+        im = fma(aim[m], vm[2 * m], im);
+      }
+      wre[0] = re;
+      wim[0] = im;
+    }
+    dst[k * ES_OUT] = make_double2(wre[0], wim[0]);
+  }
+  template <int ES_IN = 1, int ES_OUT = 1>
+  __device__ __forceinline__ void apply(const V* src, V* dst) const {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) element<ES_IN, ES_OUT>(src, dst, k);
   }
 };
 
@@ -864,7 +983,7 @@ template <int NE_IN, int ROWS_OUT>
 struct PairF64Op {
   using V = double2;
   using BArg = double;
-  static constexpr int kFixCols = 0;
+  static constexpr int kFixCols = 0, kMinCtas = 0;
   static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
   static constexpr bool kRowSplit = true;
   // b[j] split once per thread, as lane pairs for the two terms of each (m, l):
@@ -967,7 +1086,7 @@ struct PairF64Op {
 struct PairAnOp {
   using V = double2;
   using BArg = double;
-  static constexpr int kFixCols = 0;
+  static constexpr int kFixCols = 0, kMinCtas = 0;
   static constexpr int kNeIn = 9, kNeOut = 9;
   static constexpr bool kRowSplit = false;  // row k of a^dagger b reads column k of a
   PairF64Op<9, 3> pair;                     // b as FP32 pairs and the row routine
@@ -1001,7 +1120,7 @@ template <bool ADJ>
 struct PairMatVecOp {
   using V = double2;
   using BArg = double;
-  static constexpr int kFixCols = 0;
+  static constexpr int kFixCols = 0, kMinCtas = 0;
   static constexpr int kNeIn = 9, kNeOut = 3;
   static constexpr bool kRowSplit = false;  // one output vector per link
   float2 ya[3], yb[3], yla[3], ylb[3];      // v[m]: (re, im), (-im, re), and their low parts
@@ -1048,7 +1167,7 @@ template <int NE_IN, int ROWS_OUT>
 struct HybridF64Op {
   using V = double2;
   using BArg = double;
-  static constexpr int kFixCols = 3;
+  static constexpr int kFixCols = 3, kMinCtas = 0;
   static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
   static constexpr bool kRowSplit = true;
   NativeOp<kF64, NE_IN, ROWS_OUT> nat;

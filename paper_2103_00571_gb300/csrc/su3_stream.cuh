@@ -101,7 +101,7 @@ __device__ __forceinline__ int tile_link_base(int q) {
 // instead of 4,694). The other ops run faster, or as fast, with the registers it takes by itself
 // (0: not stated).
 template <class Op, int TPL, int LAYOUT, bool PADDED>
-__global__ void __launch_bounds__(256, Op::kFixCols > 0 ? 1 : 0) su3_aos_kernel(const __grid_constant__ AosArgs<typename Op::BArg> p,
+__global__ void __launch_bounds__(256, Op::kMinCtas) su3_aos_kernel(const __grid_constant__ AosArgs<typename Op::BArg> p,
                                                       const __grid_constant__ SiteMaps maps) {
   using V = typename Op::V;
   using BA = typename Op::BArg;
@@ -452,6 +452,12 @@ static su3_status run_aos(const Form& f, const LaunchCfg& cfg_in, const void* a,
   if (LAYOUT == SU3_LAYOUT_SOA && ts > kSoaPlaneLinks / 4) {
     *ctx.err = "SOA tiles hold at most 64 sites (256 links per element plane)";
     return SU3_ERR_INVALID_ARG;
+  }
+  // matrix x vector: the output ring must fit beside the input stages that suit the product, so
+  // stages go before the tile shrinks. Not in place, S stages hold S loads in flight (in place S - 1).
+  if (!kInPlace && Op::kNeOut < Op::kNeIn && ctx.smem_per_sm > 0) {
+    const long long per_cta = ctx.smem_per_sm / cfg.ctas_per_sm - ctx.smem_reserved;
+    while (cfg.stages > 2 && smem_of(ts) > per_cta) --cfg.stages;
   }
   if (LAYOUT != SU3_LAYOUT_SOA) {
     // the two-row -> full form shares its configuration with two-row -> two-row but also needs a

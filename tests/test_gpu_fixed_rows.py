@@ -125,3 +125,33 @@ def test_rows_in_every_layout(layout, ri, ro):
                            cfg=dict(block=128, tile_sites=32, stages=3, threads_per_link=tpl))
             assert np.array_equal(got, base), (V, tpl)
     h.close()
+
+
+@pytest.mark.parametrize("name", ["random", "graded", "real", "dyadic", "b_identity"])
+def test_adjacent_products(name):
+    """a^dagger b, a v and a^dagger v: the same bounds, with a's columns (conjugated) as rows."""
+    import torch
+    V = 777
+    a, b = family(name, V, np.random.default_rng(12))
+    h = su3.Handle(0)
+    d = su3.Desc(su3.F64, su3.FULL18, su3.AOS, V)
+    at = a.reshape(-1, 3, 3, 2).transpose(0, 2, 1, 3) * [1.0, -1.0]
+    dev = torch.from_numpy(a).cuda()
+    out = torch.empty_like(dev)
+    h.mult_op(su3.OP_AN, d, dev, b, d, out)
+    h.sync()
+    want, bound, _ = exact_and_bound(at.reshape(-1), b)
+    assert np.all(np.abs(out.cpu().numpy().astype(np.longdouble) - want) <= bound)
+    v = b.reshape(4, 3, 3, 2)[:, :, 0].copy()  # the first column of each matrix
+    for adjoint, rows in ((False, a), (True, at)):
+        want, _, chain = exact_and_bound(np.ascontiguousarray(rows).reshape(-1), b)
+        bv = np.zeros((4, 3, 3, 2))
+        bv[:, :, 0] = v
+        _, bound, _ = exact_and_bound(np.ascontiguousarray(rows).reshape(-1), bv.reshape(-1))
+        w = torch.zeros(V * 24, dtype=torch.float64, device="cuda")
+        h.mat_vec(d, dev, v, w, adjoint=adjoint)
+        h.sync()
+        pick = lambda x: x.reshape(-1, 3, 3, 2)[:, :, 0].reshape(-1)  # noqa: E731
+        err = np.abs(w.cpu().numpy().astype(np.longdouble) - pick(want))
+        assert np.all(err <= pick(bound)), (name, adjoint)
+    h.close()
