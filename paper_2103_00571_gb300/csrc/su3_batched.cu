@@ -124,8 +124,11 @@ __device__ __forceinline__ void batch_tile_compute_pair(unsigned char* in, int n
   }
 }
 
+// Launch bounds: one thread per link runs fastest with the registers that a stated minimum of one CTA
+// lets the compiler take (144 instead of 136: 96 lattices 0.567 -> 0.517 ms, FP64 in FP32 pairs the
+// same), one thread per row with those it takes by itself (118; 0.751 ms with 132).
 template <int TPL>
-__global__ void __launch_bounds__(256) su3_batched_kernel(const __grid_constant__ BatchArgs p) {
+__global__ void __launch_bounds__(256, TPL == 1 ? 1 : 0) su3_batched_kernel(const __grid_constant__ BatchArgs p) {
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);
   TileInfo* info = reinterpret_cast<TileInfo*>(smem + 128);
@@ -219,8 +222,9 @@ __global__ void __launch_bounds__(256) su3_batched_kernel(const __grid_constant_
 }
 
 BatchCfg default_batch_cfg() {
-  // measured best on GB300 for the 96-lattice FP64/FP32 mix (and for its FP32-pair variant):
-  // four 64-thread CTAs per SM, 32-site (18 KB) stages, three deep
+  // measured best on GB300 for the 96-lattice FP64/FP32 mix (0.517 ms) and for its FP32-pair variant
+  // (0.443 ms): four 64-thread CTAs per SM, 32-site (18 KB) stages, three deep. 128 threads with one
+  // per row: 0.517 and 0.468 ms
   BatchCfg c;
   c.block = 64;
   c.tile_sites = 32;

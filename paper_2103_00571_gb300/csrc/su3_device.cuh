@@ -220,37 +220,35 @@ struct Storage<kBF16> {
 // The four b matrices by value in a kernel's parameter block: b[j][row][col][re/im], plus the
 // constant 1.0 that FP32-pair arithmetic multiplies by (see dot_pair2: as a kernel parameter its
 // value is unknown to the compiler, so no multiply can be folded into the FMA that uses it).
-template <typename A>
+// COLS > 0 (ops with kFixCols): with b of that many columns in fixed point for FP64 rows.
+template <typename A, int COLS>
 struct BMat {
   A v[72];
   float unit;
-};
-template <>
-struct BMat<double> {
-  double v[72];
-  float unit;
   FixedMat fix;
 };
+template <typename A>
+struct BMat<A, 0> {
+  A v[72];
+  float unit;
+};
 
-// COLS: columns of the FP64 product's b for the fixed-point form (0: the op does not use it).
 template <typename A, int COLS>
-inline BMat<A> make_b(const double* b) {
-  BMat<A> m;
+inline BMat<A, COLS> make_b(const double* b) {
+  BMat<A, COLS> m;
   for (int i = 0; i < 72; ++i) m.v[i] = (A)b[i];
   m.unit = 1.0f;
-  if constexpr (sizeof(A) == 8) {
+  if constexpr (COLS > 0) {
     memset(&m.fix, 0, sizeof(m.fix));
-    if constexpr (COLS > 0) {
-      m.fix.range = fix_b<COLS>(b, m.fix.fx, m.fix.eb) ? kFixExpRange : 0;
-      m.fix.k = fixed_const();
-    }
+    m.fix.range = fix_b<COLS>(b, m.fix.fx, m.fix.eb) ? kFixExpRange : 0;
+    m.fix.k = fixed_const();
   }
   return m;
 }
 
 // Stages b (72 reals) in shared memory and lets each thread's op take its direction j = tid % 4.
 template <class Op>
-__device__ __forceinline__ void load_b_op(const BMat<typename Op::BArg>& b, typename Op::BArg* bsh, Op& op,
+__device__ __forceinline__ void load_b_op(const BMat<typename Op::BArg, Op::kFixCols>& b, typename Op::BArg* bsh, Op& op,
                                           int native_warps) {
   for (int i = threadIdx.x; i < 72; i += blockDim.x) bsh[i] = b.v[i];
   __syncthreads();

@@ -24,7 +24,7 @@ namespace su3 {
 
 constexpr int kHostTileSites = 8;  // sites per warp tile: 32 links, one per lane
 
-template <typename A>
+template <typename A, int COLS>
 struct HostArgs {
   const unsigned char* a;  // device-usable address of a in host memory
   unsigned char* c;
@@ -32,7 +32,7 @@ struct HostArgs {
   long long a_stride;  // bytes between sites
   long long c_stride;
   int native_warps;
-  BMat<A> b;
+  BMat<A, COLS> b;
 };
 
 __device__ __forceinline__ double2 ld_stream_16(const void* p) {
@@ -42,7 +42,7 @@ __device__ __forceinline__ double2 ld_stream_16(const void* p) {
 }
 
 template <class Op>
-__global__ void __launch_bounds__(256) su3_host_kernel(const __grid_constant__ HostArgs<typename Op::BArg> p) {
+__global__ void __launch_bounds__(256) su3_host_kernel(const __grid_constant__ HostArgs<typename Op::BArg, Op::kFixCols> p) {
   using V = typename Op::V;
   constexpr int NE_IN = Op::kNeIn, NE_OUT = Op::kNeOut;
   constexpr bool kInPlace = (NE_OUT == NE_IN);
@@ -91,7 +91,7 @@ static su3_status run_host(const Form& f, const LaunchCfg& cfg, const void* a, c
   constexpr bool kInPlace = (Op::kNeOut == Op::kNeIn);
   const int block = 256;
   const size_t smem = (size_t)(block / 32) * kHostTileSites * 4 * sizeof(V) * (Op::kNeIn + (kInPlace ? 0 : Op::kNeOut));
-  HostArgs<typename Op::BArg> p;
+  HostArgs<typename Op::BArg, Op::kFixCols> p;
   p.a = static_cast<const unsigned char*>(a);
   p.c = static_cast<unsigned char*>(c);
   p.n_sites = f.n_sites;

@@ -40,7 +40,7 @@
 
 namespace su3 {
 
-template <typename A>
+template <typename A, int COLS>
 struct AosArgs {
   const unsigned char* a;
   unsigned char* c;
@@ -58,7 +58,7 @@ struct AosArgs {
   int a_padded;       // AOS: a's sites are wider than their links; tiles arrive through SiteMaps::a
   int c_padded;       // AOS: c's sites are wider than their links; tiles leave through SiteMaps::c
   int soa_tensor;     // SOA: a tile's element planes move as one 2-D tensor copy each way
-  BMat<A> b;
+  BMat<A, COLS> b;
 };
 
 // Tensor maps of a and c for the TMA engine: padded AOS arrays (rows = sites, a row = the site's
@@ -101,7 +101,7 @@ __device__ __forceinline__ int tile_link_base(int q) {
 // instead of 4,694). The other ops run faster, or as fast, with the registers it takes by itself
 // (0: not stated).
 template <class Op, int TPL, int LAYOUT, bool PADDED>
-__global__ void __launch_bounds__(256, Op::kMinCtas) su3_aos_kernel(const __grid_constant__ AosArgs<typename Op::BArg> p,
+__global__ void __launch_bounds__(256, Op::kMinCtas) su3_aos_kernel(const __grid_constant__ AosArgs<typename Op::BArg, Op::kFixCols> p,
                                                       const __grid_constant__ SiteMaps maps) {
   using V = typename Op::V;
   using BA = typename Op::BArg;
@@ -319,13 +319,13 @@ __global__ void __launch_bounds__(256, Op::kMinCtas) su3_aos_kernel(const __grid
 
 // ---- SOA / AOSOA32: direct coalesced loads ----------------------------------------------------
 
-template <typename A>
+template <typename A, int COLS>
 struct DirectArgs {
   const void* a;
   void* c;
   long long n_links;
   int native_warps;       // HYBRID: warps [0, native_warps) of every CTA compute natively
-  BMat<A> b;
+  BMat<A, COLS> b;
 };
 
 template <int LAYOUT, int NE>
@@ -335,7 +335,7 @@ __device__ __forceinline__ long long elem_index(long long q, int e, long long n_
 }
 
 template <class Op, int LAYOUT, int LPT>
-__global__ void __launch_bounds__(256) su3_direct_kernel(const __grid_constant__ DirectArgs<typename Op::BArg> p) {
+__global__ void __launch_bounds__(256) su3_direct_kernel(const __grid_constant__ DirectArgs<typename Op::BArg, Op::kFixCols> p) {
   using V = typename Op::V;
   constexpr int NE_IN = Op::kNeIn, NE_OUT = Op::kNeOut;
   __shared__ typename Op::BArg bsh[72];
@@ -486,7 +486,7 @@ static su3_status run_aos(const Form& f, const LaunchCfg& cfg_in, const void* a,
       cfg.block = (int)std::min<long long>(cfg.block, std::max<long long>(32, (items + 31) / 32 * 32));
     }
   }
-  AosArgs<BA> p;
+  AosArgs<BA, Op::kFixCols> p;
   p.a = static_cast<const unsigned char*>(a);
   p.c = static_cast<unsigned char*>(c);
   p.n_sites = f.n_sites;
@@ -558,7 +558,7 @@ static su3_status run_aos(const Form& f, const LaunchCfg& cfg_in, const void* a,
 template <class Op, int LAYOUT>
 static su3_status run_direct(const Form& f, const LaunchCfg& cfg, const void* a, const double* b, void* c,
                              const LaunchCtx& ctx) {
-  DirectArgs<typename Op::BArg> p;
+  DirectArgs<typename Op::BArg, Op::kFixCols> p;
   p.a = a;
   p.c = c;
   p.n_links = 4 * f.n_sites;
