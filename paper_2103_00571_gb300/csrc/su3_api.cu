@@ -178,11 +178,11 @@ su3_status check_cfg(su3_handle* h, const Form& f, const LaunchCfg& c) {
 }
 
 // The configuration of the (a, c) repr pair, else that of a's repr in and out, else the default.
-LaunchCfg cfg_for(su3_handle* h, const su3_desc* d, const Form& f) {
+LaunchCfg cfg_for(su3_handle* h, const su3_desc* d, const Form& f, bool adjacent = false) {
   auto it = h->cfgs.find(form_key(d, f.repr_out));
   if (it == h->cfgs.end() && f.repr_out != d->repr) it = h->cfgs.find(form_key(d));
   if (it != h->cfgs.end()) return it->second;
-  return default_cfg(f);
+  return adjacent ? default_adjacent_cfg(f) : default_cfg(f);
 }
 
 // Validates an (a, c) descriptor pair into a Form.
@@ -503,7 +503,7 @@ su3_status su3_mult_op(su3_handle* h, int32_t op, const su3_desc* a_desc, const 
     return fail(h, SU3_ERR_INVALID_ARG, "a and c overlap without being the same array");
   }
   if (h->fault & kFaultLaunch) return fail(h, SU3_ERR_FAULT_INJECTED, "fault injected at launch");
-  LaunchCfg cfg = cfg_for(h, a_desc, f);
+  LaunchCfg cfg = cfg_for(h, a_desc, f, true);
   cfg.threads_per_link = 1;  // row k of a^dagger b reads column k of a: no row split
   s = check_cfg(h, f, cfg);
   if (s != SU3_OK) return s;
@@ -529,7 +529,7 @@ su3_status su3_mat_vec(su3_handle* h, int32_t adjoint, const su3_desc* a_desc, c
   if (ranges_overlap(a_dev, su3_array_bytes(a_desc), w_dev, f.n_sites * f.c_stride))
     return fail(h, SU3_ERR_INVALID_ARG, "a and w overlap");
   if (h->fault & kFaultLaunch) return fail(h, SU3_ERR_FAULT_INJECTED, "fault injected at launch");
-  LaunchCfg cfg = cfg_for(h, a_desc, f);
+  LaunchCfg cfg = cfg_for(h, a_desc, f, true);
   cfg.threads_per_link = 1;  // one output vector per link
   s = check_cfg(h, f, cfg);
   if (s != SU3_OK) return s;

@@ -52,6 +52,8 @@ inline int64_t link_bytes(int dtype, int repr) { return (int64_t)n_elem(repr) * 
 
 // Default launch configuration of a form (used until the autotuner sets one).
 LaunchCfg default_cfg(const Form& f);
+// The same for su3_mult_op's a^dagger b and su3_mat_vec.
+LaunchCfg default_adjacent_cfg(const Form& f);
 
 // HYBRID: warps per CTA on the FP64 pipe, the nearest to native_permille of the CTA's warps.
 inline int native_warps(const Form& f, const LaunchCfg& cfg) {

@@ -33,31 +33,62 @@ su3_status launch_selftest_wait(int limit_ms, const LaunchCtx& ctx) {
 
 // ---- host launchers -----------------------------------------------------------------------------
 
-LaunchCfg default_cfg(const Form& f) {
-  LaunchCfg c;
-  if (f.layout == SU3_LAYOUT_AOS) {
-    c.block = 128;
-    // ~18 KB per tile for FP64 full sites, ~9-18 KB for the narrower forms
-    const int64_t site_in = f.a_stride;
-    int ts = (int)std::max<int64_t>(32, std::min<int64_t>(128, 18432 / std::max<int64_t>(site_in, 1)));
-    c.tile_sites = ts;
-    c.stages = 4;
-    c.ctas_per_sm = 2;
-    if (f.dtype == SU3_F64 && f.arith == SU3_ARITH_NATIVE) {
-      // four CTAs of four warps: 5,220 GB/s at 2^21 sites (4 stages x 2 CTAs: half the warps, 3.1 TB/s)
-      c.tile_sites = 32;
-      c.stages = 3;
-      c.ctas_per_sm = 4;
-    }
-  } else {
-    c.block = 256;
-    c.tile_sites = f.dtype == SU3_F64 ? 1 : f.dtype == SU3_F32 ? 2 : 4;  // links per thread
-    c.stages = 0;
-    c.ctas_per_sm = 4;
+// The AOS shape that suits every form somewhat: ~18 KB per tile for FP64 full sites, 9-18 KB for the
+// narrower ones, in 8 warps per SM. It divides small and middling arrays more evenly than larger tiles do.
+static LaunchCfg general_cfg(const Form& f) {
+  const int tile = (int)std::max<int64_t>(32, std::min<int64_t>(128, 18432 / std::max<int64_t>(f.a_stride, 1)));
+  return LaunchCfg{128, tile, 4, 2, 0, 1};
+}
+
+// The shapes that measured best (block, sites per tile, stages, CTAs per SM, threads per link); GB/s at
+// 48^4 sites, in brackets those of general_cfg.
+static LaunchCfg measured_cfg(const Form& f) {
+  const bool two_in = f.repr_in == SU3_REPR_TWOROW12, two_out = f.repr_out == SU3_REPR_TWOROW12;
+  const bool narrow = f.dtype == SU3_F16 || f.dtype == SU3_BF16;
+  const long long n = f.n_sites > 0 ? f.n_sites : 1ll << 36;  // a form without a size: the large shape
+  auto cfg = [](int block, int tile, int stages, int ctas, int tpl) {
+    return LaunchCfg{block, tile, stages, ctas, 0, tpl};
+  };
+  if (f.layout != SU3_LAYOUT_AOS) {
+    // direct loads, AOSOA32 (256 threads, 4 CTAs, 1/2/4 links for 16/8/4-byte elements before): FP64
+    // 5,050 (4,223), FP32 6,717 (6,333), two-row FP32 6,668 (6,222), FP16 6,426 (6,389), two-row
+    // FP16 6,407 (5,468)
+    if (f.dtype == SU3_F64) return f.arith == SU3_ARITH_NATIVE ? cfg(128, 1, 0, 16, 1) : cfg(256, 1, 0, 4, 1);
+    if (narrow) return two_out ? cfg(128, 2, 0, 8, 1) : cfg(128, 4, 0, 4, 1);
+    return two_out ? cfg(128, 2, 0, 4, 1) : cfg(256, 2, 0, 8, 1);
   }
+  if (f.dtype == SU3_F64 && f.arith == SU3_ARITH_NATIVE) {
+    if (two_out) return cfg(128, 48, 3, 4, 3);  // 5,030: 16 warps, rows as work items
+    if (two_in) return cfg(128, 48, 3, 3, 1);   // 2,770: 152 registers
+    return cfg(128, 32, 3, 4, 1);               // 5,355: 16 warps of 124 registers
+  }
+  if (f.dtype == SU3_F64) {  // FP32 pairs
+    if (two_in) return cfg(128, 64, 3, 3, 1);                   // 5,683 (3,758); to full 4,430 (3,194)
+    return n >= 1 << 18 ? cfg(128, 32, 3, 4, 1) : general_cfg(f);  // 5,906 (4,716); level at 10^5 sites
+  }
+  if (two_in != two_out) return general_cfg(f);
+  if (f.dtype == SU3_F32) {
+    if (two_out) return cfg(256, 96, 6, 1, 3);                     // 6,940 (6,010)
+    return n >= 1 << 20 ? cfg(64, 128, 4, 1, 1) : general_cfg(f);  // 6,951 (6,339); 14.7 (10.6) us at 10^5 sites
+  }
+  return two_out ? general_cfg(f) : cfg(128, 64, 6, 3, 3);  // FP16 6,639 (5,790); two-row level
+}
+
+// The adjacent products: their FP64 forms take the product's shapes (a^dagger b 4,590, a v 6,139 GB/s);
+// the narrower storage types, which have no row split here, the general one (FP16 a^dagger b 6,210 GB/s, 5,840
+// in the product's shape).
+LaunchCfg default_adjacent_cfg(const Form& f) { return f.dtype == SU3_F64 ? default_cfg(f) : general_cfg(f); }
+
+LaunchCfg default_cfg(const Form& f) {
+  LaunchCfg c = measured_cfg(f);
+  // a tile's sites may span 1 MiB of the array; wide strides keep tiles of 32 sites
+  if (f.layout == SU3_LAYOUT_AOS)
+    c.tile_sites = (int)std::min<int64_t>(c.tile_sites, std::max<int64_t>(32, (1 << 20) / std::max<int64_t>(f.a_stride, 1)));
   c.native_permille = f.arith == SU3_ARITH_HYBRID ? 125 : 0;
   if (f.arith == SU3_ARITH_HYBRID) {
     c.block = 256;  // 8 warps, one of them native
+    c.threads_per_link = 1;
+    c.ctas_per_sm = f.layout == SU3_LAYOUT_AOS ? 2 : 4;
     if (f.layout == SU3_LAYOUT_AOS) {
       c.tile_sites = 64;  // 256 links: one per thread and tile
       c.stages = 3;       // two such CTAs fit in one SM's shared memory
