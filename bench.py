@@ -53,7 +53,7 @@ def parse():
     ap.add_argument("--L", type=int, default=64)
     ap.add_argument("--quick", action="store_true", help="headline only: no forms/batched/e2e/cpu legs")
     ap.add_argument("--arith", default="native", choices=["native", "f32pair", "hybrid"],
-                    help="arithmetic of the FP64 AoS step (native = the plain FP64 method)")
+                    help="arithmetic of the FP64 AoS step (native = FP64 accuracy)")
     ap.add_argument("--dtype", default="f64", choices=["f64", "f32", "f16", "bf16"],
                     help="storage type of the timed step (other than f64: with --quick, for profiling)")
     ap.add_argument("--stride", type=int, default=0,
@@ -481,7 +481,9 @@ def run_native(args, world, rank, local):
     # roofline of the dominant kernel (the FP64 AoS kernel is the whole step); its template's
     # threads per link: 1, or 3 when the launch splits links into rows
     tpl = 3 if h.get_launch_cfg_for(d64, dc)["threads_per_link"] == 3 else 1
-    fp64_peak = sms * 2 * 2 * sm_max * 1e6 / 1e12  # 2 DFMA/clk/SM x 2 flop x clock, TFLOP/s
+    # The FP64 product's peak, TFLOP/s by the paper's count: the FP64 pipe's 2 FMA per clock and SM beside
+    # the integer units' 32 wide multiply-adds, of which 18 make the 6 FMAs of one output real
+    fp64_peak = sms * (2 * 2 + 32 / 18 * 6 * 2) * sm_max * 1e6 / 1e12
     flop_site = flop_per_site(d64.repr, dc.repr)
     achieved_tf = flop_site * V / (per_launch_ms * 1e-3) / 1e12
     achieved_gbs = bytes_per_step / (per_launch_ms * 1e-3) / 1e9
@@ -509,12 +511,15 @@ def run_native(args, world, rank, local):
         roofline = {"bound": "alu", "achieved": round(achieved_tf, 4), "peak": round(fp64_peak, 4),
                     "unit": "TFLOP/s", "frac": round(achieved_tf / fp64_peak, 4), "traffic": traffic,
                     "kernel": "su3_aos_kernel<NativeOp<F64,%s>, %d, AOS, %s>" % (ops, tpl, padded),
-                    "peak_source": "FP64 pipe: %d SMs (this device) x 2 DFMA/clk x 2 flop x %.0f MHz (max SM clock)"
+                    "peak_source": "%d SMs (this device) x %.0f MHz (max SM clock) x (FP64 pipe 2 DFMA/clk x 2 flop + "
+                                   "integer units 32 wide multiply-adds/clk, 18 for the 12 flop of an output real)"
                                        % (sms, sm_max),
                     "peak_measured": round(fp64_measured, 4) if fp64_measured else None,
                     "frac_of_measured": round(achieved_tf / fp64_measured, 4) if fp64_measured else None,
-                    "peak_measured_source": "su3_measure_fp64_rate: 8 independent DFMA chains per thread, "
-                                            "2,048 threads per SM, CUDA events",
+                    "peak_measured_source": "FP64 pipe alone (five of six output reals are computed in fixed point on "
+                                            "the integer units, so the fraction passes 1): su3_measure_fp64_rate, 8 "
+                                            "independent DFMA chains per thread, 2,048 threads per SM, CUDA events",
+                    "arithmetic": "FP64 FMAs, and 61-bit fixed point with one rounding (half the error on random SU(3))",
                     "hbm": hbm_roof}
     else:
         tr = traffic_record().get("su3_aos_kernel<f64,full,%s%s>" % (args.arith, pad), {})

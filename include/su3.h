@@ -90,8 +90,7 @@ typedef enum { SU3_LAYOUT_AOS = 0, SU3_LAYOUT_AOSOA32 = 1, SU3_LAYOUT_SOA = 2 } 
 typedef enum { SU3_ARITH_NATIVE = 0, SU3_ARITH_F32PAIR = 1, SU3_ARITH_HYBRID = 2 } su3_arith;
 /*
  * SU3_ARITH_HYBRID (F64 storage): in every CTA the first round(native_permille/1000 * warps) warps
- * compute their links with NATIVE FP64 FMAs on the FP64 pipe while the other warps use F32PAIR on
- * the FP32 pipe, so both pipes work at once. Each link's result is exactly what NATIVE or F32PAIR
+ * compute their links with NATIVE arithmetic while the other warps use F32PAIR on the FP32 pipe. Each link's result is exactly what NATIVE or F32PAIR
  * would produce for it; accuracy is that of F32PAIR. Same repr and range rules as F32PAIR.
  */
 
