@@ -59,7 +59,7 @@ static LaunchCfg measured_cfg(const Form& f) {
   }
   if (f.dtype == SU3_F64 && f.arith == SU3_ARITH_NATIVE) {
     if (two_out) return cfg(128, 48, 3, 4, 3);  // 5,030: 16 warps, rows as work items
-    if (two_in) return cfg(128, 48, 3, 3, 1);   // 2,770: 152 registers
+    if (two_in) return cfg(64, 24, 3, 6, 1);    // 3,060: 152 registers, 12 warps (128 x 48 x 3 CTAs 2,880)
     return cfg(128, 32, 3, 4, 1);               // 5,355: 16 warps of 124 registers
   }
   if (f.dtype == SU3_F64) {  // FP32 pairs
