@@ -485,6 +485,7 @@ def run_native(args, world, rank, local):
     # the integer units' 32 wide multiply-adds, of which 18 make the 6 FMAs of one output real
     fp64_peak = sms * (2 * 2 + 32 / 18 * 6 * 2) * sm_max * 1e6 / 1e12
     flop_site = flop_per_site(d64.repr, dc.repr)
+    fp64_share = 1 / 6 if d64.repr == dc.repr else 192 / flop_site  # of the flops, on the FP64 pipe
     achieved_tf = flop_site * V / (per_launch_ms * 1e-3) / 1e12
     achieved_gbs = bytes_per_step / (per_launch_ms * 1e-3) / 1e9
     try:  # the FP64 pipe's sustained rate, measured on this device by a diagnostic FMA kernel
@@ -515,9 +516,9 @@ def run_native(args, world, rank, local):
                                    "integer units 32 wide multiply-adds/clk, 18 for the 12 flop of an output real)"
                                        % (sms, sm_max),
                     "peak_measured": round(fp64_measured, 4) if fp64_measured else None,
-                    "frac_of_measured": round(achieved_tf / fp64_measured, 4) if fp64_measured else None,
-                    "peak_measured_source": "FP64 pipe alone (five of six output reals are computed in fixed point on "
-                                            "the integer units, so the fraction passes 1): su3_measure_fp64_rate, 8 "
+                    "frac_of_measured": round(achieved_tf * fp64_share / fp64_measured, 4) if fp64_measured else None,
+                    "peak_measured_source": "the FP64 pipe alone, and the share of the flops that it does (one output "
+                                            "real of six, or row 2's rebuild) against it: su3_measure_fp64_rate, 8 "
                                             "independent DFMA chains per thread, 2,048 threads per SM, CUDA events",
                     "arithmetic": "FP64 FMAs, and 61-bit fixed point with one rounding (half the error on random SU(3))",
                     "hbm": hbm_roof}
