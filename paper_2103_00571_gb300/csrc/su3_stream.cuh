@@ -482,8 +482,14 @@ static su3_status run_aos(const Form& f, const LaunchCfg& cfg_in, const void* a,
     t2 = std::max(quantum, (t2 + quantum - 1) / quantum * quantum);
     if (t2 < ts) {
       ts = t2;
+      // FP64 in fixed point: one thread per output row while a tile's rows fit one CTA, since a whole
+      // link is a chain of three rows (per launch at 64 sites 5.8 -> 3.7 us, 1,000 sites 5.9 -> 4.3,
+      // 2,000 sites 5.3 -> 4.7; with more rows than threads, at 4,096 sites, 5.5 either way)
+      const bool split = kInPlace && Op::kRowSplit && Op::kFixCols > 0 && f.arith == SU3_ARITH_NATIVE &&
+                         ts * 4 * (Op::kNeOut / 3) <= 256;
+      if (split) cfg.threads_per_link = 3;
       const long long items = ts * 4 * (cfg.threads_per_link == 1 ? 1 : (Op::kRowSplit ? Op::kNeOut / 3 : 1));
-      cfg.block = (int)std::min<long long>(cfg.block, std::max<long long>(32, (items + 31) / 32 * 32));
+      cfg.block = (int)std::min<long long>(split ? 256 : cfg.block, std::max<long long>(32, (items + 31) / 32 * 32));
     }
   }
   AosArgs<BA, Op::kFixCols> p;
