@@ -66,13 +66,15 @@ typedef enum { SU3_REPR_FULL18 = 0, SU3_REPR_TWOROW12 = 1 } su3_repr;
 typedef enum { SU3_LAYOUT_AOS = 0, SU3_LAYOUT_AOSOA32 = 1, SU3_LAYOUT_SOA = 2 } su3_layout;
 
 /*
- * Arithmetic of the F64 storage type. NATIVE: FP64 accuracy (the plain method's results). a x b
- * is computed by FP64 fused multiply-adds and, beside them, in 61-bit fixed point on the integer
- * units with one rounding per result: off by at most half an ulp + 5 * 2^-58 of (the largest real
- * of the row of a) x (the largest real of b[j]), each rounded up to a power of two, for rows and
- * matrices whose reals are of similar size; the others (zeros, reals spread over many binary
- * orders, extreme or non-finite values) by FP64 FMAs throughout. On random SU(3) matrices that is
- * half the error of FP64 FMAs alone.
+ * Arithmetic of the F64 storage type. NATIVE: FP64 accuracy. Every result is within the bound of six
+ * FP64 fused multiply-adds, 6 * 2^-53 * S, S the sum of its own six |a||b|, and products and sums that
+ * FP64 holds (of integers, as a rule) are exact. The results are not those of a chain of FMAs bit for
+ * bit: where S is at least 1/16 of (the largest real of the row of a) x (the largest real of b[j]), each
+ * rounded up to a power of two, five results of six come from 61-bit fixed point on the integer units
+ * with one rounding, off by at most 2^-53 |c| + 1.9 * 2^-53 * S; the others (rows with zeros, reals
+ * spread over more than 2^31, extreme or non-finite values, and all rows when b has few reals near its
+ * largest) by FP64 FMAs. On random SU(3) matrices the error is half that of FP64 FMAs alone. Calls
+ * whose values keep to the FMAs run at their speed, about 0.3 of the other's.
  * F32PAIR: FP64 storage, arithmetic on unevaluated pairs of FP32 numbers. Each a element is split
  * into hi + lo with integer operations; each output real is a compensated dot product (TwoSum on
  * the running FP32 sum, the product error and the product's share of the TwoSum error added by one
@@ -248,7 +250,7 @@ su3_status su3_mult_batched(su3_handle* h, int32_t n, const su3_batch_item* item
  * pool or fixed memory budget, and loops that must never stall, since cudaMalloc/cudaFree can
  * synchronise the whole device. Those callers cannot create a handle either (su3_init allocates),
  * so this entry point takes none and allocates nothing: the lattice descriptors go into a
- * statically allocated device area of 256 + SU3_STATIC_MAX_LATTICES * 1192 bytes (about 298 KB),
+ * statically allocated device area of 256 + SU3_STATIC_MAX_LATTICES * 1328 bytes (about 332 KB),
  * which every GPU that loads libsu3 holds until the process exits.
  *  - Runs on the calling thread's current CUDA device. The first call on each device looks up the
  *    area's device address (set-up, once per device); make that first call before any stream

@@ -90,14 +90,22 @@ __device__ __forceinline__ void batch_tile_compute(unsigned char* in, int nt, co
   }
 }
 
-// FP64 lattice: rows in fixed point (the op of the single-lattice kernels, so the same bits).
+// FP64 lattice: rows in fixed point (the op of the single-lattice kernels, so the same bits). b's words
+// are in registers: with few warps per SM, reading them from the descriptor for each row took 0.584 ms
+// for 96 lattices, 0.560 so.
 template <int TPL>
 __device__ __forceinline__ void batch_tile_compute_f64(unsigned char* in, int nt, const BatchDesc& d,
                                                        const FixedConst& k) {
   const int j = threadIdx.x & 3;
   NativeOp<kF64, 9, 3> op;
   op.init(d.b + 18 * j, 0);
-  op.fix.take(d.bfix[j], d.eb[j], d.fixed ? kFixExpRange : 0, k);
+  int4 fx[9];
+  uint4 mg[2];
+#pragma unroll
+  for (int e = 0; e < 9; ++e) fx[e] = reinterpret_cast<const int4*>(d.bfix[j])[e];
+  mg[0] = reinterpret_cast<const uint4*>(d.bmag[j])[0];
+  mg[1] = reinterpret_cast<const uint4*>(d.bmag[j])[1];
+  op.fix.take(fx, mg, d.eb[j], d.fixed ? kFixExpRange : 0, k);
   const int links = 4 * nt;
   for (int q = threadIdx.x; q < TPL * links; q += blockDim.x) {
     int row, link;
@@ -125,8 +133,8 @@ __device__ __forceinline__ void batch_tile_compute_pair(unsigned char* in, int n
 }
 
 // Launch bounds: one thread per link runs fastest with the registers that a stated minimum of one CTA
-// lets the compiler take (144 instead of 136: 96 lattices 0.567 -> 0.517 ms, FP64 in FP32 pairs the
-// same), one thread per row with those it takes by itself (118; 0.751 ms with 132).
+// lets the compiler take (184 instead of 142: 96 lattices 0.593 -> 0.560 ms, FP64 in FP32 pairs 0.473 ->
+// 0.449), one thread per row with those it takes by itself.
 template <int TPL>
 __global__ void __launch_bounds__(256, TPL == 1 ? 1 : 0) su3_batched_kernel(const __grid_constant__ BatchArgs p) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -222,9 +230,9 @@ __global__ void __launch_bounds__(256, TPL == 1 ? 1 : 0) su3_batched_kernel(cons
 }
 
 BatchCfg default_batch_cfg() {
-  // measured best on GB300 for the 96-lattice FP64/FP32 mix (0.517 ms) and for its FP32-pair variant
-  // (0.443 ms): four 64-thread CTAs per SM, 32-site (18 KB) stages, three deep. 128 threads with one
-  // per row: 0.517 and 0.468 ms
+  // measured on GB300 for the 96-lattice FP64/FP32 mix (0.560 ms) and for its FP32-pair variant
+  // (0.449 ms): four 64-thread CTAs per SM, 32-site (18 KB) stages, three deep. 128 threads with one
+  // per row: 0.548 and 0.472 ms
   BatchCfg c;
   c.block = 64;
   c.tile_sites = 32;
@@ -307,7 +315,7 @@ su3_status launch_batched(const BatchDesc* descs_dev, int n, int total_tiles, co
 
 namespace su3 {
 
-static_assert(sizeof(BatchDesc) == 1192, "the static area's documented size assumes 1192-byte descriptors");
+static_assert(sizeof(BatchDesc) == 1328, "the static area's documented size assumes 1328-byte descriptors");
 constexpr size_t kStaticHeader = 256;
 constexpr size_t kStaticBytes = kStaticHeader + (size_t)SU3_STATIC_MAX_LATTICES * sizeof(BatchDesc);
 

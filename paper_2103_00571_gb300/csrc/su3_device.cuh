@@ -240,21 +240,40 @@ inline BMat<A, COLS> make_b(const double* b) {
   m.unit = 1.0f;
   if constexpr (COLS > 0) {
     memset(&m.fix, 0, sizeof(m.fix));
-    m.fix.range = fix_b<COLS>(b, m.fix.fx, m.fix.eb) ? kFixExpRange : 0;
+    m.fix.range = fix_b<COLS>(b, m.fix.fx, m.fix.mag, m.fix.eb) ? kFixExpRange : 0;
     m.fix.k = fixed_const();
   }
   return m;
 }
 
-// Stages b (72 reals) in shared memory and lets each thread's op take its direction j = tid % 4.
+// b in shared memory: its 72 reals, and with COLS > 0 (FP64 rows in fixed point) fix_b's words.
+template <typename A, int COLS>
+struct BShared {
+  alignas(16) A v[72];
+  int fx[4][9][4];
+  unsigned mag[4][kFixMags];
+};
+template <typename A>
+struct BShared<A, 0> {
+  A v[72];
+};
 template <class Op>
-__device__ __forceinline__ void load_b_op(const BMat<typename Op::BArg, Op::kFixCols>& b, typename Op::BArg* bsh, Op& op,
+using BSharedOf = BShared<typename Op::BArg, Op::kFixCols>;
+
+// Stages b in shared memory and lets each thread's op take its direction j = tid % 4.
+template <class Op>
+__device__ __forceinline__ void load_b_op(const BMat<typename Op::BArg, Op::kFixCols>& b, BSharedOf<Op>* bsh, Op& op,
                                           int native_warps) {
-  for (int i = threadIdx.x; i < 72; i += blockDim.x) bsh[i] = b.v[i];
+  for (int i = threadIdx.x; i < 72; i += blockDim.x) bsh->v[i] = b.v[i];
+  if constexpr (Op::kFixCols > 0) {
+    for (int i = threadIdx.x; i < 4 * 9 * 4; i += blockDim.x) (&bsh->fx[0][0][0])[i] = (&b.fix.fx[0][0][0])[i];
+    for (int i = threadIdx.x; i < 4 * kFixMags; i += blockDim.x) (&bsh->mag[0][0])[i] = (&b.fix.mag[0][0])[i];
+  }
   __syncthreads();
-  op.init(bsh + 18 * (threadIdx.x & 3), native_warps);
+  const int j = threadIdx.x & 3;
+  op.init(bsh->v + 18 * j, native_warps);
   op.set_unit(b.unit);
-  if constexpr (Op::kFixCols > 0) op.set_fixed(b.fix, threadIdx.x & 3);
+  if constexpr (Op::kFixCols > 0) op.set_fixed(b.fix, bsh->fx[j], bsh->mag[j], j);
 }
 
 // ---- the link product -------------------------------------------------------------------------
@@ -352,54 +371,47 @@ __device__ __forceinline__ void link_mult(const Link<T>& a, const T (&bre)[9], c
 // One output row takes 36 FP64 FMAs, of which GB300 does 2 per clock and SM: by themselves they
 // hold the FP64 product at 24 % of the memory bandwidth, with every other unit idle. The integer
 // units do 32 multiply-adds of 32 x 32 + 64 bits per clock and SM beside them. So five of a row's
-// six output reals are computed in fixed point, at FP64 accuracy, while the FP64 pipe computes the
-// sixth:
+// six output reals are computed in fixed point while the FP64 pipe computes the sixth:
 //  * a's row becomes 61-bit fixed point relative to its largest real, A = ah * 2^32 + al with a
 //    29-bit ah and a sign, and al a signed 32-bit limb; b comes from the host in the same form
 //    (fix_b). A real within 2^-8 of the largest is exact; a smaller one is cut at 2^-61 of it.
 //  * an output is the sum of six products A * B: H = sum ah*bh, X = sum ah*bl and Y = sum al*bh,
 //    in 64-bit accumulators that cannot overflow (6 * 2^58, 6 * 2^60), and T = H + X/2^32 + Y/2^32.
-//    al*bl is left out (below 1.5 units of T). The start values make X and Y unsigned
-//    (xbias = 2^63), so that their high words need no sign extension, and take that 2 * 2^31 back
-//    and round (hbias).
+//    al*bl is left out (below 1.5 units of T). X and Y start at 2^63 + 2^31 (xbias): unsigned, their
+//    high words need no sign extension, and they are rounded; hbias takes the 2 * 2^31 back.
 //  * T becomes a double with one rounding (fixed_to_f64).
-// T's unit is 2^-58 of (the row's largest real) x (b's), each rounded up to a power of two. T is off
-// by at most 5 units (al*bl 1.5, the two shifts 1, a's cut 0.75 and its negation 0.4, b's rounding
-// 0.4, T's one's complement 1), as a rule by 0.5. So an output is within half an ulp + 5 * 2^-58 of
-// that product. Over random SU(3) matrices the error is 2.5e-17 of the result's norm, 4.7e-17 with
-// every sixth output by FMAs, against 9.8e-17 for FMAs alone; the largest single error 3.3e-16
-// against 4.4e-16.
-// The bound does not shrink with the terms, so a row whose terms may all be small takes FP64 FMAs
-// throughout. b is checked by fix_b. In a row, at least four of the six reals must be within 2^-8
-// of the largest: ensured by the exponents' distances from the largest summing to at most 26
-// (three above 8 would make 27), which costs an add per real. With three of b's reals in every
-// column within 2^-5, every output then has a term of at least 2^-14 of T's full scale. 99.98 % of
-// the rows of random SU(3) matrices pass (with a limit of 23, 99.92 %: 4 % slower). Rows with
-// zeros, subnormals, infinities or NaN, or outside 2^-723 .. 2^677, do not pass. Which way a row
-// goes depends on its values only, so results are the same for every launch shape and layout.
-// Measured (AOS, 2^21 sites): FP64 FMAs alone 1,585 GB/s; six outputs of six in fixed point 4,711,
-// five 5,220 (the multiplier 55 %, FP64 pipe 60 % and ALU 45 % busy; a wide multiply-add holds
-// back the other integer pipe, so they do not overlap fully), 14 of 18 5,187, 13 of 18 4,869, 12
-// of 18 4,273.
+// T's unit is 2^-58 of full scale, (the row's largest real) x (b's), each rounded up to a power of
+// two. T is off by at most 3.7 units (al*bl 1.5, X and Y 0.5 each, a's cut 0.75, b's rounding 0.4),
+// as a rule by 0.5. Limbs of zero make no error: products of few enough bits for FP64 FMAs to be
+// exact (integers, as a rule) are exact here too.
+// The 3.7 units do not shrink with the terms, so every output real passes a gate: the sum S of its six
+// |a||b| must be 1/16 of full scale, and is not in 1 of 10^5 of random SU(3) matrices. Then 3.7 units
+// are at most 1.9 * 2^-53 S, and the output is off by at most 2^-53 |c| + 1.9 * 2^-53 S, against 6 *
+// 2^-53 S for six FMAs; over the matrices tried (random and near the identity, reals spread over
+// up to 31 binary orders, integers) at most 1.6 * 2^-53 S against 4.7, r.m.s. 0.24 to 0.42 against 0.45
+// to 0.79. S is estimated from below by two dot products of bytes, from |a| cut to 5 bits and |b| to 8.
+// An output real that does not pass, or is below 2^-26 of full scale (not normalised), is computed by
+// FP64 FMAs; so are all of a row whose reals are spread over more than 2^31 (any zero), not finite or
+// outside 2^-723 .. 2^677, and all rows when fix_b refuses b. Which way an output goes depends on its
+// row's and b's values only, so results are the same for every launch shape and layout.
+// Measured (AOS, 48^4 sites, GB/s): FP64 FMAs alone 1,585; random SU(3) 5,128, 5,395 without the
+// gate; links exp(i e H) at e = 0.05 2,952; an identity or real a or b 1,575. The wide multiply-adds
+// and the other integer instructions share their issue, so they set the rate (364 instructions per
+// row, 90 of them wide multiply-adds). 4 of 18 output reals on the FP64 pipe instead of 3: 4,916.
+// b is read from shared memory for each row: in registers 4,869, at 124 of them instead of 112. S in FP32,
+// on the idle half of the FP32 pipe: 4,739.
 
-// b[j] (or v[j]) of one thread as fixed-point limbs: element 3*m + l (COLS 3) or m (COLS 1).
+// b[j] (or v[j]) of one thread in fixed point, in memory: element e = 3*m + l (COLS 3) or m (COLS 1).
 template <int COLS>
 struct FixedB {
-  int rh[3 * COLS], rl[3 * COLS], ih[3 * COLS], il[3 * COLS];
+  const int4* limbs;  // (re_hi, re_lo, im_hi, im_lo)
+  const uint4* mags;  // fix_b's magnitudes, two words per column
   unsigned kb, range;
   FixedConst k;
-  // from fix_b's limbs of b[j] (8-byte aligned), its exponent, and the exponents of a's rows taken
-  __device__ __forceinline__ void take(const int (*fx)[4], int eb, unsigned exp_range, const FixedConst& c) {
-    const int2* p = reinterpret_cast<const int2*>(fx);
-#pragma unroll
-    for (int e = 0; e < 3 * COLS; ++e) {
-      const int2 r = p[2 * e], i = p[2 * e + 1];
-      rh[e] = r.x;
-      rl[e] = r.y;
-      ih[e] = i.x;
-      il[e] = i.y;
-    }
-    kb = (unsigned)(1085 - 1080 + eb) << 20;
+  __device__ __forceinline__ void take(const void* fx, const void* mag, int eb, unsigned exp_range, const FixedConst& c) {
+    limbs = static_cast<const int4*>(fx);
+    mags = static_cast<const uint4*>(mag);
+    kb = (unsigned)(1085 - 1080 - 31 + eb) << 20;
     range = exp_range;
     k = c;
   }
@@ -419,28 +431,29 @@ __device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
   return d;
 }
 
-// T in units of 2^k as a double, rounded once to nearest (ties away from zero); `base` is
-// (1023 + 62 + k) << 20. Valid while |T|'s high word is not 0: `least` collects its minimum. The
-// magnitude is T's one's complement when T is negative: one unit of T less, far below the rounding.
-__device__ __forceinline__ double fixed_to_f64(long long t, unsigned base, unsigned& least) {
+// T in units of 2^k as a double, rounded once to nearest; `base` is (1054 + k) << 20. Valid while |T|'s
+// high word is not 0; else `bad` gets bits above the low five. A negative T is worked on as its one's
+// complement, shifted with ones: one unit of its 63 normalised bits below |T|, which only turns a tie.
+__device__ __forceinline__ double fixed_to_f64(long long t, unsigned base, unsigned& bad) {
   int th, tl;
   asm("mov.b64 {%0, %1}, %2;" : "=r"(tl), "=r"(th) : "l"(t));
   const int s = th >> 31;
   const unsigned ah = (unsigned)(th ^ s), al = (unsigned)(tl ^ s);
-  least = min(least, ah);
-  unsigned n, mh, ml, lo, hi;
-  asm("clz.b32 %0, %1;" : "=r"(n) : "r"(ah));
-  asm("shf.l.wrap.b32 %0, %1, %2, %3;" : "=r"(mh) : "r"(al), "r"(ah), "r"(n));
-  asm("shl.b32 %0, %1, %2;" : "=r"(ml) : "r"(al), "r"(n));
-  asm("shf.r.wrap.b32 %0, %1, %2, 11;" : "=r"(lo) : "r"(ml), "r"(mh));
-  hi = mh >> 11;  // with the leading bit, which adds the last 1 to the exponent field
-  const unsigned e = (base | ((unsigned)s & 0x80000000u)) - (n << 20);
-  asm("{add.cc.u32 %0, %0, %2; addc.u32 %1, %1, %3;}" : "+r"(lo), "+r"(hi) : "r"((ml >> 10) & 1u), "r"(e));
+  unsigned p, mh, ml, lo, hi;
+  asm("bfind.u32 %0, %1;" : "=r"(p) : "r"(ah));  // ~0 for 0
+  bad |= p;
+  const unsigned n = p + 2;
+  asm("shf.r.wrap.b32 %0, %1, %2, %3;" : "=r"(mh) : "r"(al), "r"(ah), "r"(n));
+  asm("shf.r.wrap.b32 %0, %1, %2, %3;" : "=r"(ml) : "r"(s), "r"(al), "r"(n));
+  asm("{add.cc.u32 %0, %0, 0x200; addc.u32 %1, %1, 0;}" : "+r"(ml), "+r"(mh));
+  asm("shf.r.wrap.b32 %0, %1, %2, 10;" : "=r"(lo) : "r"(ml), "r"(mh));
+  hi = (mh >> 10) + ((base | ((unsigned)th & 0x80000000u)) + (p << 20));
   return __hiloint2double((int)hi, (int)lo);
 }
 
-// Whether a row (reals a[0..2].re, a[0..2].im) suits the fixed-point form: the distances d of its
-// exponents from the largest, each at most 26, and e0 = 0x7ff - the largest exponent field.
+// A row's exponents (reals a[0..2].re, a[0..2].im): their distances d from the largest, and e0 = 0x7ff -
+// the largest exponent field. The row suits the fixed-point form when take() is true and spread() has
+// no bit above the low five.
 struct FixedExps {
   int d[6], e0;
   __device__ __forceinline__ bool take(const double (&are)[3], const double (&aim)[3], unsigned range) {
@@ -452,44 +465,75 @@ struct FixedExps {
     }
     const unsigned lowest = min(min(min(hn[0], hn[1]), min(hn[2], hn[3])), min(hn[4], hn[5]));
     e0 = (int)(lowest >> 20);
-    int sum = 0;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      d[q] = (int)(hn[q] >> 20) - e0;
-      sum += d[q];
-    }
-    return sum <= 26 && (unsigned)(0x7ff - kFixExpMin) - (unsigned)e0 < range;
+    for (int q = 0; q < 6; ++q) d[q] = (int)(hn[q] >> 20) - e0;
+    return (unsigned)(0x7ff - kFixExpMin) - (unsigned)e0 < range;
   }
+  __device__ __forceinline__ unsigned spread() const { return (unsigned)(d[0] | d[1] | d[2] | d[3] | d[4] | d[5]); }
 };
 
-// One output row c[l] = sum_m a[m] b[m][l], l < COLS, of a row whose exponents suit; bj = the same b
-// in FP64 (re, im of element COLS*m + l). The last NAT (0 or 1) output reals by FP64 FMAs, in
-// row_mult's order. Returns false, with c undefined, when a result is too small for the form.
+// Output real `out` = 2*l + (0 re, 1 im) of the row a[] times column l of b, by FP64 FMAs in row_mult's
+// order; bj = b[j] in FP64 (re, im of element COLS*m + l).
+template <int COLS>
+__device__ __forceinline__ double fma_output(const double (&are)[3], const double (&aim)[3], const double* bj, int out) {
+  const int l = out >> 1, im = out & 1;
+  double c = are[0] * bj[2 * l + im];
+  c = fma(im ? aim[0] : -aim[0], bj[2 * l + 1 - im], c);
+#pragma unroll
+  for (int m = 1; m < 3; ++m) {
+    c = fma(are[m], bj[2 * (COLS * m + l) + im], c);
+    c = fma(im ? aim[m] : -aim[m], bj[2 * (COLS * m + l) + 1 - im], c);
+  }
+  return c;
+}
+
+// The output reals of a row but for the last NAT: c[2*l] = re and c[2*l + 1] = im of sum_m a[m] b[m][l],
+// l < COLS. Returns the set (bit 2*l + im) of those that FP64 FMAs have to do instead.
 template <int COLS, int NAT>
-__device__ __forceinline__ bool fixed_row(const double (&are)[3], const double (&aim)[3], const FixedExps& ex,
-                                          const FixedB<COLS>& b, const double* bj, double (&cre)[COLS],
-                                          double (&cim)[COLS]) {
-  const double x[6] = {are[0], are[1], are[2], aim[0], aim[1], aim[2]};
-  int ah[6], al[6];
+__device__ __forceinline__ unsigned fixed_row(const double (&are)[3], const double (&aim)[3], const FixedExps& ex,
+                                              const FixedB<COLS>& b, double (&c)[2 * COLS]) {
+  constexpr int kOut = 2 * COLS - NAT;
+  int ah[6], al[6], nh[3], nl[3];  // limbs of re, im and -im
+  unsigned mag[6];                 // the magnitudes' high words: 29 bits
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
-    const int h = __double2hiint(x[q]);
-    const unsigned l = (unsigned)__double2loint(x[q]);
-    const unsigned s = (unsigned)(h >> 31);
+    const double x = q < 3 ? are[q % 3] : aim[q % 3];
+    const int h = __double2hiint(x);
+    const unsigned l = (unsigned)__double2loint(x);
     const unsigned m = ((unsigned)h & 0xfffffu) | b.k.lead;
-    const unsigned wh = __funnelshift_l(l, m, 8) ^ s, wl = (l << 8) ^ s;
-    const unsigned vl = __funnelshift_r(wl, wh, ex.d[q]);
-    ah[q] = ((int)wh >> ex.d[q]) + (int)(vl >> 31);
+    const unsigned w = __funnelshift_l(l, m, 8), s = (unsigned)(h >> 31);
+    mag[q] = w >> ex.d[q];
+    unsigned vh = mag[q] ^ s, vl = __funnelshift_r(l << 8, w, ex.d[q]) ^ s;
+    asm("{sub.cc.u32 %0, %0, %2; subc.u32 %1, %1, %2;}" : "+r"(vl), "+r"(vh) : "r"(s));
+    ah[q] = (int)(vh + (vl >> 31));
     al[q] = (int)vl;
+    if (q >= 3) {
+      asm("{sub.cc.u32 %0, %2, %0; subc.u32 %1, %2, %1;}" : "+r"(vl), "+r"(vh) : "r"(b.k.zero));
+      nh[q - 3] = (int)(vh + (vl >> 31));
+      nl[q - 3] = (int)vl;
+    }
   }
-  int nh[3], nl[3];  // of -im (-al less one unit: al may be -2^31)
+  // the gate: |re|, |im| of elements 0 and 1, then of 2, in bytes of 1/32 of full scale; im's sums take
+  // them the other way round
+  const unsigned r01 = __byte_perm(__byte_perm(mag[0], mag[3], 0x0073), __byte_perm(mag[1], mag[4], 0x0073), 0x5410);
+  const unsigned r2 = __byte_perm(mag[2], mag[5], 0x0073);  // b's bytes 2 and 3 are 0 here
+  const unsigned i01 = __byte_perm(r01, 0, 0x2301), i2 = __byte_perm(r2, 0, 0x2301);
+  unsigned bm[(2 * COLS + 3) / 4 * 4], rest = 0;
 #pragma unroll
-  for (int m = 0; m < 3; ++m) {
-    nh[m] = b.k.zero - ah[3 + m];
-    nl[m] = al[3 + m] ^ b.k.ones;
+  for (int i = 0; i < (2 * COLS + 3) / 4; ++i) {
+    const uint4 v = b.mags[i];
+    bm[4 * i] = v.x;
+    bm[4 * i + 1] = v.y;
+    bm[4 * i + 2] = v.z;
+    bm[4 * i + 3] = v.w;
+  }
+#pragma unroll
+  for (int o = kOut - 1; o >= 0; --o) {
+    const unsigned sum = __dp4a(o & 1 ? i2 : r2, bm[o | 1], 0u - kFixMinSum);
+    rest = __funnelshift_l(__dp4a(o & 1 ? i01 : r01, bm[o & ~1], sum), rest, 1);  // its sign
   }
   const unsigned base = ((0x7ffu - (unsigned)ex.e0) << 20) + b.kb;
-  unsigned least = 0x7fffffffu;
+  unsigned bad = ex.spread();
   auto sum3 = [](long long h, long long u, long long v) {
     return h + (long long)((unsigned long long)u >> 32) + (long long)((unsigned long long)v >> 32);
   };
@@ -499,38 +543,49 @@ __device__ __forceinline__ bool fixed_row(const double (&are)[3], const double (
     long long hr = b.k.hbias, xr = b.k.xbias, yr = b.k.xbias, hi = b.k.hbias, xi = b.k.xbias, yi = b.k.xbias;
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-      const int e = COLS * m + l;
-      hr = mad_wide(ah[m], b.rh[e], hr);
-      hr = mad_wide(nh[m], b.ih[e], hr);
-      xr = mad_wide(ah[m], b.rl[e], xr);
-      xr = mad_wide(nh[m], b.il[e], xr);
-      yr = mad_wide(al[m], b.rh[e], yr);
-      yr = mad_wide(nl[m], b.ih[e], yr);
-      if (l < COLS - NAT) {
-        hi = mad_wide(ah[m], b.ih[e], hi);
-        hi = mad_wide(ah[3 + m], b.rh[e], hi);
-        xi = mad_wide(ah[m], b.il[e], xi);
-        xi = mad_wide(ah[3 + m], b.rl[e], xi);
-        yi = mad_wide(al[m], b.ih[e], yi);
-        yi = mad_wide(al[3 + m], b.rh[e], yi);
+      const int4 w = b.limbs[COLS * m + l];
+      hr = mad_wide(ah[m], w.x, hr);
+      hr = mad_wide(nh[m], w.z, hr);
+      xr = mad_wide(ah[m], w.y, xr);
+      xr = mad_wide(nh[m], w.w, xr);
+      yr = mad_wide(al[m], w.x, yr);
+      yr = mad_wide(nl[m], w.z, yr);
+      if (2 * l + 1 < kOut) {
+        hi = mad_wide(ah[m], w.z, hi);
+        hi = mad_wide(ah[3 + m], w.x, hi);
+        xi = mad_wide(ah[m], w.w, xi);
+        xi = mad_wide(ah[3 + m], w.y, xi);
+        yi = mad_wide(al[m], w.z, yi);
+        yi = mad_wide(al[3 + m], w.x, yi);
       }
     }
-    const long long tr = sum3(hr, xr, yr), ti = sum3(hi, xi, yi);
-    cre[l] = fixed_to_f64(tr, base, least);
-    if (l < COLS - NAT) {
-      cim[l] = fixed_to_f64(ti, base, least);
-    } else {
-      double im = are[0] * bj[2 * l + 1];
-      im = fma(aim[0], bj[2 * l], im);
-#pragma unroll
-      for (int m = 1; m < 3; ++m) {
-        im = fma(are[m], bj[2 * (COLS * m + l) + 1], im);
-        im = fma(aim[m], bj[2 * (COLS * m + l)], im);
-      }
-      cim[l] = im;
-    }
+    c[2 * l] = fixed_to_f64(sum3(hr, xr, yr), base, bad);
+    if (2 * l + 1 < kOut) c[2 * l + 1] = fixed_to_f64(sum3(hi, xi, yi), base, bad);
   }
-  return least != 0;  // a result below 2^-27 of the row's largest times b's: FP64 FMAs
+  return bad & ~31u ? ~0u : rest;
+}
+
+// A whole row c = a b (c as in fixed_row): its output reals in fixed point where that suits, the last
+// NAT and the others by FP64 FMAs. bj = b[j] in FP64.
+template <int COLS, int NAT>
+__device__ __forceinline__ void row_f64(const double (&are)[3], const double (&aim)[3], const FixedB<COLS>& b,
+                                        const double* bj, double (&c)[2 * COLS]) {
+  constexpr int kOut = 2 * COLS - NAT;
+  unsigned rest = ~0u;
+  FixedExps ex;
+  if (ex.take(are, aim, b.range)) {
+    rest = fixed_row<COLS, NAT>(are, aim, ex, b, c);
+#pragma unroll
+    for (int o = kOut; o < 2 * COLS; ++o) c[o] = fma_output<COLS>(are, aim, bj, o);
+  } else {
+#pragma unroll
+    for (int o = kOut; o < 2 * COLS; ++o) c[o] = fma_output<COLS>(are, aim, bj, o);
+  }
+  if (rest) {
+#pragma unroll
+    for (int o = 0; o < kOut; ++o)
+      if (rest >> o & 1) c[o] = fma_output<COLS>(are, aim, bj, o);
+  }
 }
 
 // ---- per-link operations used by the streaming kernels ----------------------------------------
@@ -600,7 +655,7 @@ struct NativeOp<kF64, NE_IN, ROWS_OUT> {
   using V = double2;
   using BArg = double;
   static constexpr int kFixCols = 3;
-  static constexpr int kMinCtas = 1;
+    static constexpr int kMinCtas = NE_IN == 6 && ROWS_OUT == 3 ? 1 : 2;
   static constexpr int kNeIn = NE_IN, kNeOut = 3 * ROWS_OUT;
   static constexpr bool kRowSplit = true;
   // output reals per row on the FP64 pipe; two-row in, full out has its rebuild of row 2 there
@@ -610,24 +665,24 @@ struct NativeOp<kF64, NE_IN, ROWS_OUT> {
   __device__ __forceinline__ void begin_tile(int) {}
   __device__ __forceinline__ void set_unit(float) {}
   __device__ __forceinline__ void init(const BArg* bj, int /*native_warps*/) { bm = bj; }
-  __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { fix.take(f.fx[j], f.eb[j], f.range, f.k); }
+  __device__ __forceinline__ void set_fixed(const FixedMat& f, const void* fx, const void* mag, int j) {
+    fix.take(fx, mag, f.eb[j], f.range, f.k);
+  }
   __device__ __forceinline__ void row(const double (&are)[3], const double (&aim)[3], double (&cre)[3],
                                       double (&cim)[3]) const {
-    FixedExps ex;
-    if (ex.take(are, aim, fix.range) && fixed_row<3, kNat>(are, aim, ex, fix, bm, cre, cim)) return;
-    double bre[9], bim[9];
+    double c[6];
+    row_f64<3, kNat>(are, aim, fix, bm, c);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      bre[e] = bm[2 * e];
-      bim[e] = bm[2 * e + 1];
+    for (int l = 0; l < 3; ++l) {
+      cre[l] = c[2 * l];
+      cim[l] = c[2 * l + 1];
     }
-    row_mult(are, aim, bre, bim, cre, cim);
   }
   template <int ES_IN = 1, int ES_OUT = 1>
   __device__ __forceinline__ void apply(const V* src, V* dst) const {
     if constexpr (NE_IN == 6 && ROWS_OUT == 3) {
       // two-row in, full out (never in place): row 2 is rebuilt first, so that the FP64 pipe works on
-      // it beside rows 0 and 1 (2,886 against 2,825 GB/s at L=48; the same operations as apply_row, so
+      // it beside rows 0 and 1 (2,937 against 2,878 GB/s at L=48; the same operations as apply_row, so
       // the same bits)
       double r0re[3], r0im[3], r1re[3], r1im[3], r2re[3], r2im[3], cre[3], cim[3];
 #pragma unroll
@@ -770,7 +825,7 @@ struct MatVecOp {  // w[k] = sum_m a[k][m] v[m]   (ADJ: sum_m conj(a[m][k]) v[m]
 // The same for FP64 storage, rows in fixed point (fixed_row): row k of a^dagger b is the conjugate of
 // a's column k times b, and an element of a v is a's row k times the one column v (all in fixed point:
 // with one of six on the FP64 pipe a^dagger v measured 9 % slower). At L=48, FP64 FMAs before:
-// a^dagger b 1,568 -> 4,590 GB/s, a v 2,960 -> 6,139, a^dagger v 2,950 -> 5,648 (the products' launch shape).
+// a^dagger b 1,568 -> 4,836 GB/s, a v 2,960 -> 5,566, a^dagger v 2,950 -> 5,246 (the products' launch shape).
 template <>
 struct AnOp<kF64> {
   using V = double2;
@@ -783,7 +838,9 @@ struct AnOp<kF64> {
   __device__ __forceinline__ void begin_tile(int) {}
   __device__ __forceinline__ void set_unit(float) {}
   __device__ __forceinline__ void init(const BArg* bj, int w) { op.init(bj, w); }
-  __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { op.set_fixed(f, j); }
+  __device__ __forceinline__ void set_fixed(const FixedMat& f, const void* fx, const void* mag, int j) {
+    op.set_fixed(f, fx, mag, j);
+  }
   template <int ES_IN = 1, int ES_OUT = 1>
   __device__ __forceinline__ void apply(const V* src, V* dst) const {
     double2 a[9];  // all of a first: the output may overwrite it (in place)
@@ -817,30 +874,20 @@ struct MatVecOp<kF64, ADJ> {
   __device__ __forceinline__ void begin_tile(int) {}
   __device__ __forceinline__ void set_unit(float) {}
   __device__ __forceinline__ void init(const BArg* vj, int) { vm = vj; }
-  __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { fix.take(f.fx[j], f.eb[j], f.range, f.k); }
+  __device__ __forceinline__ void set_fixed(const FixedMat& f, const void* fx, const void* mag, int j) {
+    fix.take(fx, mag, f.eb[j], f.range, f.k);
+  }
   template <int ES_IN, int ES_OUT>
   __device__ __forceinline__ void element(const V* src, V* dst, int k) const {
-    double are[3], aim[3], wre[1], wim[1];
+    double are[3], aim[3], w[2];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       const double2 x = src[(ADJ ? 3 * m + k : 3 * k + m) * ES_IN];
       are[m] = x.x;
       aim[m] = ADJ ? -x.y : x.y;
     }
-    FixedExps ex;
-    if (!(ex.take(are, aim, fix.range) && fixed_row<1, 0>(are, aim, ex, fix, vm, wre, wim))) {
-      double re = 0, im = 0;
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        re = fma(are[m], vm[2 * m], re);
-        re = fma(-aim[m], vm[2 * m + 1], re);
-        im = fma(are[m], vm[2 * m + 1], im);
-        im = fma(aim[m], vm[2 * m], im);
-      }
-      wre[0] = re;
-      wim[0] = im;
-    }
-    dst[k * ES_OUT] = make_double2(wre[0], wim[0]);
+    row_f64<1, 0>(are, aim, fix, vm, w);
+    dst[k * ES_OUT] = make_double2(w[0], w[1]);
   }
   template <int ES_IN = 1, int ES_OUT = 1>
   __device__ __forceinline__ void apply(const V* src, V* dst) const {
@@ -1183,7 +1230,9 @@ struct HybridF64Op {
     native = period > 0 && ((k + (int)(threadIdx.x >> 5)) % period) == 0;
   }
   __device__ __forceinline__ void set_unit(float u) { pair.set_unit(u); }
-  __device__ __forceinline__ void set_fixed(const FixedMat& f, int j) { nat.set_fixed(f, j); }
+  __device__ __forceinline__ void set_fixed(const FixedMat& f, const void* fx, const void* mag, int j) {
+    nat.set_fixed(f, fx, mag, j);
+  }
   template <int ES_IN = 1, int ES_OUT = 1>
   __device__ __forceinline__ void apply(const V* src, V* dst) const {
     if (native) nat.template apply<ES_IN, ES_OUT>(src, dst);

@@ -53,9 +53,9 @@ __global__ void __launch_bounds__(256) su3_host_kernel(const __grid_constant__ H
   constexpr int kSlot = kHostTileSites * (kSiteIn + (kInPlace ? 0 : kSiteOut));
 
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ typename Op::BArg bsh[72];
+  __shared__ BSharedOf<Op> bsh;
   Op op;
-  load_b_op(p.b, bsh, op, p.native_warps);  // the only CTA barrier
+  load_b_op(p.b, &bsh, op, p.native_warps);  // the only CTA barrier
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   unsigned char* in = smem + (size_t)warp * kSlot;

@@ -89,32 +89,40 @@ su3_status launch_unpack(const Form& src, const void* src_dev, double* dst, cons
 // products by -x into negated multiplies and splits multiply-accumulates into a product and 64-bit
 // adds (19 more integer adds per output: 4,142 against 4,732 GB/s at 2^21 sites).
 struct FixedConst {
-  int zero, ones;          // 0, -1
+  int zero;
   unsigned lead;           // 2^20: the implicit leading bit of an FP64 mantissa, in its high word
   long long hbias, xbias;  // start values of the accumulators
 };
-inline FixedConst fixed_const() { return FixedConst{0, -1, 1u << 20, 1 - (1ll << 32), (long long)(1ull << 63)}; }
+inline FixedConst fixed_const() {
+  return FixedConst{0, 1u << 20, -(1ll << 32), (long long)((1ull << 63) + (1ull << 31))};
+}
+
+// Biased exponents of a row's largest |real| that the form takes: 2^-723 <= |a| < 2^677.
+constexpr unsigned kFixExpMin = 300, kFixExpRange = 1400;
+// Least sum of the |a||b| of an output real's six terms, in 2^-13 of full scale: 1/16 (fixed_row).
+constexpr unsigned kFixMinSum = 512;
+// Words per direction of fix_b's magnitudes: 6, padded to 16-byte words.
+constexpr int kFixMags = 8;
 
 // Element e of b[j] as two signed 32-bit limbs for re and two for im, fx[j][e] = (re_hi, re_lo,
 // im_hi, im_lo), value (hi * 2^32 + lo) * 2^(eb[j] - 61) with |b[j]| < 2^eb[j]. `range`: the number of
 // exponents of a row's largest real that the fixed-point form takes, 0 when b does not suit it.
 struct FixedMat {
-  alignas(8) int fx[4][9][4];
+  alignas(16) int fx[4][9][4];
+  unsigned mag[4][kFixMags];
   int eb[4];
   unsigned range;
   FixedConst k;
 };
 
-// Biased exponents of a row's largest |real| that the form takes: 2^-723 <= |a| < 2^677.
-constexpr unsigned kFixExpMin = 300, kFixExpRange = 1400;
-
-// Fills fx and eb from b (COLS 3: [j][row][col]; 1: one colour vector per j at the start of b's j-th
-// 18 reals). Returns whether b suits the form: every value finite, the largest of each matrix within
-// 1e-30 .. 1e30, and in every column at least three of the six reals within 2^-5 of that largest
-// (see fixed_row for why). 99.9 % of sets of four random SU(3) matrices do; when one matrix does not,
-// every row takes FP64 FMAs.
+// Fills fx, mag (column l: |re| and |im| of rows 0 and 1 in bytes of 2^(eb - 8), then of row 2) and eb
+// from b (COLS 3: [j][row][col]; 1: one colour vector per j at the start of b's j-th 18 reals). Returns
+// whether b suits the form: every value finite, the largest of each matrix within 1e-30 .. 1e30, and
+// in every column at least three of the six reals within 2^-5 of that largest, since with fewer most
+// output reals would not pass fixed_row's gate. 99.9 % of sets of four random SU(3) matrices do; when one
+// matrix does not, every row takes FP64 FMAs.
 template <int COLS>
-inline bool fix_b(const double* b, int (*fx)[9][4], int* eb) {
+inline bool fix_b(const double* b, int (*fx)[9][4], unsigned (*mag)[kFixMags], int* eb) {
   for (int j = 0; j < 4; ++j) {
     const double* m = b + 18 * j;
     double top = 0;
@@ -131,12 +139,19 @@ inline bool fix_b(const double* b, int (*fx)[9][4], int* eb) {
         for (int c = 0; c < 2; ++c) n += fabs(m[2 * (COLS * r + l) + c]) >= large;
       if (n < 3) return false;
     }
-    const double scale = ldexp(1.0, 61 - eb[j]);
+    const double scale = ldexp(1.0, 61 - eb[j]), bytes = ldexp(1.0, 8 - eb[j]);
     for (int q = 0; q < 6 * COLS; ++q) {
       const long long v = (long long)rint(m[q] * scale);
       const int lo = (int)(unsigned)((unsigned long long)v & 0xffffffffull);
       fx[j][q >> 1][2 * (q & 1)] = (int)((v - lo) >> 32);
       fx[j][q >> 1][2 * (q & 1) + 1] = lo;
+    }
+    for (int l = 0; l < COLS; ++l) {
+      unsigned w[3];  // an element's |re| and |im| as bytes, rounded down
+      for (int r = 0; r < 3; ++r)
+        w[r] = (unsigned)(fabs(m[2 * (COLS * r + l)]) * bytes) | (unsigned)(fabs(m[2 * (COLS * r + l) + 1]) * bytes) << 8;
+      mag[j][2 * l] = w[0] | w[1] << 16;
+      mag[j][2 * l + 1] = w[2];
     }
   }
   return true;
@@ -154,11 +169,13 @@ struct BatchDesc {
   signed char eb[4];   // F64 NATIVE: exponents of the four matrices (fix_b)
   double b[72];        // FP64 b (F32 lattices round it in the kernel)
   union {
-    float bpair[144];    // F32PAIR: b[j][e] split as (re_hi, im_hi, re_lo, im_lo), [j][e][4]
-    int bfix[4][9][4];   // F64 NATIVE: b in fixed point (fix_b)
+    alignas(16) float bpair[144];  // F32PAIR: b[j][e] split as (re_hi, im_hi, re_lo, im_lo), [j][e][4]
+    int bfix[4][9][4];             // F64 NATIVE: b in fixed point (fix_b)
   };
+  unsigned bmag[4][kFixMags];  // F64 NATIVE: fix_b's magnitudes
 };
-static_assert(offsetof(BatchDesc, bfix) % 8 == 0 && sizeof(BatchDesc) % 8 == 0, "bfix is read as 8-byte words");
+static_assert(offsetof(BatchDesc, bfix) % 16 == 0 && offsetof(BatchDesc, bmag) % 16 == 0 && sizeof(BatchDesc) % 16 == 0,
+              "bfix and bmag are read as 16-byte words");
 
 // Fills BatchDesc::bpair from the FP64 b (hi = b rounded to FP32, lo = the rest rounded to FP32).
 inline void split_b_pairs(const double* b, float* out) {
@@ -178,10 +195,11 @@ inline void fill_batch_b(BatchDesc* o, int dtype, int arith, const double* b) {
   o->fixed = 0;
   for (int j = 0; j < 4; ++j) o->eb[j] = 0;
   for (int i = 0; i < 72; ++i) o->b[i] = b[i];
+  for (int i = 0; i < 4 * kFixMags; ++i) (&o->bmag[0][0])[i] = 0;
   if (dtype == SU3_F64 && arith == SU3_ARITH_NATIVE) {
     int eb[4] = {0, 0, 0, 0};
     for (int i = 0; i < 144; ++i) o->bpair[i] = 0;
-    o->fixed = fix_b<3>(b, o->bfix, eb) ? 1 : 0;
+    o->fixed = fix_b<3>(b, o->bfix, o->bmag, eb) ? 1 : 0;
     for (int j = 0; j < 4; ++j) o->eb[j] = (signed char)eb[j];  // |eb| <= 101
   } else {
     split_b_pairs(b, o->bpair);

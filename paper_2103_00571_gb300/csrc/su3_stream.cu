@@ -58,9 +58,9 @@ static LaunchCfg measured_cfg(const Form& f) {
     return two_out ? cfg(128, 2, 0, 4, 1) : cfg(256, 2, 0, 8, 1);
   }
   if (f.dtype == SU3_F64 && f.arith == SU3_ARITH_NATIVE) {
-    if (two_out) return cfg(128, 48, 3, 4, 3);  // 5,030: 16 warps, rows as work items
-    if (two_in) return cfg(64, 24, 3, 6, 1);    // 3,060: 152 registers, 12 warps (128 x 48 x 3 CTAs 2,880)
-    return cfg(128, 32, 3, 4, 1);               // 5,355: 16 warps of 124 registers
+    if (two_out) return cfg(128, 48, 3, 4, 3);  // 4,977: 16 warps, rows as work items
+    if (two_in) return cfg(64, 24, 2, 6, 1);    // 2,925: 12 warps of 154 registers; with three stages they do not fit
+    return cfg(128, 32, 3, 4, 1);               // 5,094: 16 warps of 110 registers
   }
   if (f.dtype == SU3_F64) {  // FP32 pairs
     if (two_in) return cfg(128, 64, 3, 3, 1);                   // 5,683 (3,758); to full 4,430 (3,194)

@@ -70,7 +70,12 @@ struct SiteMaps {
   CUtensorMap c;
 };
 
-constexpr int kSmemHeader = 1024;    // mbarriers (<= 8 x 8 B) + b (<= 576 B), then 128-aligned data
+// Shared memory before the stages: mbarriers (<= 8 x 8 B) and b (BShared: 576 B, or 1,280 with the
+// fixed-point rows' words), then 128-aligned data.
+template <class Op>
+constexpr int smem_header() {
+  return Op::kFixCols > 0 ? 1408 : 1024;
+}
 constexpr int kSoaPlaneLinks = 256;  // links per element plane of an SOA tile in shared memory
 
 // Distance, in storage vectors, between consecutive elements of one link inside a staged tile.
@@ -96,9 +101,9 @@ __device__ __forceinline__ int tile_link_base(int q) {
 // PADDED (AOS only): a's or c's sites are wider than their links, and `maps` holds their tensor
 // maps; otherwise `maps` is read only by SOA tensor copies. One instantiation per PADDED value, so
 // the packed kernels keep their own code.
-// Launch bounds: a stated minimum of one CTA per SM lets the compiler use more registers for its
-// schedule (FP64 rows in fixed point: 124 instead of 103, 5,355 instead of 5,043 GB/s at L=48; two-row 4,993
-// instead of 4,694). The other ops run faster, or as fast, with the registers it takes by itself
+// Launch bounds: a stated minimum of two CTAs per SM lets the compiler use up to 128 registers for its
+// schedule (FP64 rows in fixed point: 110 instead of 76, 5,098 instead of 4,755 GB/s at L=48; two-row 4,863
+// instead of 4,484). The other ops run faster, or as fast, with the registers it takes by itself
 // (0: not stated).
 template <class Op, int TPL, int LAYOUT, bool PADDED>
 __global__ void __launch_bounds__(256, Op::kMinCtas) su3_aos_kernel(const __grid_constant__ AosArgs<typename Op::BArg, Op::kFixCols> p,
@@ -122,8 +127,9 @@ __global__ void __launch_bounds__(256, Op::kMinCtas) su3_aos_kernel(const __grid
 
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);
-  BA* bsh = reinterpret_cast<BA*>(smem + 64);
-  unsigned char* stage0 = smem + kSmemHeader;
+  BSharedOf<Op>* bsh = reinterpret_cast<BSharedOf<Op>*>(smem + 64);
+  static_assert(64 + sizeof(BSharedOf<Op>) <= smem_header<Op>(), "b overlaps the stages");
+  unsigned char* stage0 = smem + smem_header<Op>();
   unsigned char* out0 = stage0 + (size_t)p.stages * p.stage_bytes;
 
   const int tid = threadIdx.x;
@@ -338,10 +344,10 @@ template <class Op, int LAYOUT, int LPT>
 __global__ void __launch_bounds__(256) su3_direct_kernel(const __grid_constant__ DirectArgs<typename Op::BArg, Op::kFixCols> p) {
   using V = typename Op::V;
   constexpr int NE_IN = Op::kNeIn, NE_OUT = Op::kNeOut;
-  __shared__ typename Op::BArg bsh[72];
+  __shared__ BSharedOf<Op> bsh;
   const long long q_end = p.n_links;
   Op op;
-  load_b_op(p.b, bsh, op, p.native_warps);
+  load_b_op(p.b, &bsh, op, p.native_warps);
   const V* a = reinterpret_cast<const V*>(p.a);
   V* c = reinterpret_cast<V*>(p.c);
   const long long T = (long long)gridDim.x * blockDim.x;  // a multiple of 4: j stays tid % 4
@@ -429,7 +435,7 @@ static su3_status run_aos(const Form& f, const LaunchCfg& cfg_in, const void* a,
   const bool warp_out = !kInPlace && LAYOUT == SU3_LAYOUT_AOS && !PADDED && cfg.threads_per_link == 1 &&
                         Op::kNeIn == 6 && Op::kNeOut == 9 && kVec == 16;
   auto smem_of = [&](long long ts) {
-    return kSmemHeader + cfg.stages * in_bytes(ts) + (warp_out ? cfg.block / 32 * 2 * 32 * kLinkOut : 3 * out_bytes(ts));
+    return smem_header<Op>() + cfg.stages * in_bytes(ts) + (warp_out ? cfg.block / 32 * 2 * 32 * kLinkOut : 3 * out_bytes(ts));
   };
 
   long long ts = cfg.tile_sites;

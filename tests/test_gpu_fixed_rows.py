@@ -1,10 +1,11 @@
 """The FP64 product's fixed-point rows (NATIVE arithmetic) against extended precision, at the edges of
 their range: rows whose reals differ in size just inside and outside what the fixed-point form takes,
-zeros, extreme and non-finite values, and b matrices that suit it or do not.
+zeros, extreme and non-finite values, outputs whose terms are all small, and b matrices that suit it or
+do not.
 
-Bounds. A row in fixed point: half an ulp of the result, plus 5 units of 2^-58 of (largest real of
-the row, rounded up to a power of two) x (the same of b): the sums of the terms that are left out or
-rounded. A row by FP64 FMAs: six roundings, 6 * 2^-53 * sum |a||b|.
+Bound. Every output real, fixed point or FP64 FMAs: six roundings, 6 * 2^-53 * sum |a||b| over its own
+six terms. (In fixed point it is one rounding and 3.7 units of 2^-58 of full scale, where sum |a||b| is
+at least 1/16 of full scale: 2.9 * 2^-53 * sum |a||b|.) Products that six FMAs give exactly are exact.
 """
 import numpy as np
 import pytest
@@ -33,13 +34,7 @@ def exact_and_bound(a, b):
     ci = np.einsum("qkm,qml->qkl", ar, bi) + np.einsum("qkm,qml->qkl", ai, br)
     mag = lambda x, y, z, w: np.einsum("qkm,qml->qkl", abs(x), abs(y)) + np.einsum("qkm,qml->qkl", abs(z), abs(w))  # noqa: E731
     s = np.stack([mag(ar, br, ai, bi), mag(ar, bi, ai, br)], -1)
-    up = lambda x: 2.0 ** np.ceil(np.log2(np.where(x > 0, x, 1).astype(np.float64)))  # noqa: E731
-    top = up(np.maximum(abs(ar), abs(ai)).max(2, keepdims=True))[..., None] * up(
-        np.maximum(abs(br), abs(bi)).max((1, 2), keepdims=True))[..., None]
-    c = np.stack([cr, ci], -1)
-    fixed = U * abs(c) + 5 * 2.0 ** -58 * top
-    chain = 6 * U * s
-    return c.reshape(-1), np.maximum(fixed, chain).reshape(-1), chain.reshape(-1)
+    return np.stack([cr, ci], -1).reshape(-1), (6 * U * s).reshape(-1)
 
 
 def family(name, V, rng):
@@ -64,6 +59,22 @@ def family(name, V, rng):
     elif name == "dyadic":  # low limbs of all ones and all zeros, exact powers of two
         a = np.sign(a) * np.where(rng.random(a.size) < 0.5, 1.0 - 2.0 ** -rng.integers(1, 54, a.size),
                                   2.0 ** -rng.integers(0, 4, a.size).astype(float))
+    elif name == "small_terms":  # rows and columns whose large reals meet the small ones: sums of 2^-13
+        a = np.sign(a) * rng.uniform(1, 2, a.size)
+        a.reshape(-1, 3, 2)[:, 2, 0] *= 2.0 ** -2
+        a.reshape(-1, 3, 2)[:, :, 1] *= 2.0 ** -8
+        b = np.sign(b) * rng.uniform(1, 2, 72)
+        b.reshape(4, 3, 3, 2)[:, :, 0] *= [0.0, 2.0 ** -4]
+    elif name == "wide":  # reals of a row spread over up to 2^31, the limit of the form, and beyond
+        a = a * 2.0 ** -rng.integers(0, 34, a.size)
+    elif name == "smooth":  # links at various distances from the identity
+        a = a * np.repeat(2.0 ** -rng.integers(1, 12, V * 4), 18)
+        a.reshape(-1, 3, 3, 2)[:, range(3), range(3), 0] += 1.0
+    elif name == "one_direction":  # b = 1 links beside random ones in every warp
+        a.reshape(-1, 4, 18)[:, 0] = 0.0
+        a.reshape(-1, 4, 3, 3, 2)[:, 0, range(3), range(3), 0] = 1.0
+    elif name == "b_small":  # reals of b far below the largest of their matrix
+        b = b * 2.0 ** -rng.permutation(np.repeat(np.arange(0, 36, 6), 12))
     elif name == "b_identity":
         b = np.zeros(72)
         b.reshape(4, 3, 3, 2)[:, range(3), range(3), 0] = 1.0
@@ -75,8 +86,8 @@ def family(name, V, rng):
     return a, b
 
 
-FAMILIES = ["random", "graded", "spread", "identity", "real", "large", "small", "scaled", "dyadic", "b_identity",
-            "b_one_sparse", "b_scaled"]
+FAMILIES = ["random", "graded", "spread", "identity", "real", "large", "small", "scaled", "dyadic", "small_terms",
+            "wide", "smooth", "one_direction", "b_small", "b_identity", "b_one_sparse", "b_scaled"]
 
 
 @pytest.mark.parametrize("name", FAMILIES)
@@ -85,14 +96,51 @@ def test_error_bound(name):
     a, b = family(name, V, np.random.default_rng(11))
     h = su3.Handle(0)
     c = run_form(h, a, b, su3.F64)
-    want, bound, chain = exact_and_bound(a, b)
+    want, bound = exact_and_bound(a, b)
     err = np.abs(c.astype(np.longdouble) - want)
     assert np.all(np.isfinite(c))
     assert np.all(err <= bound + 2.0 ** -1073), name
-    if name in ("real", "identity", "large", "small", "b_identity", "b_one_sparse"):  # rows by FMAs throughout
-        assert np.all(err <= chain + 2.0 ** -1073), name
-    if name == "random":  # fixed point is the more exact: every row of FMAs measures 9.8e-17
+    if name in ("random", "b_scaled"):  # fixed point is the more exact: rows of FMAs throughout measure 9.8e-17
         assert np.linalg.norm(err.astype(float)) < 7e-17 * np.linalg.norm(want.astype(float))
+    h.close()
+
+
+def integers(shape, bits, rng):
+    return rng.integers(1, 2 ** bits, shape) * rng.choice([-1.0, 1.0], shape)
+
+
+@pytest.mark.parametrize("bits_a,bits_b", [(3, 3), (10, 10), (24, 24), (30, 3), (3, 30), (29, 20)])
+def test_integers_are_exact(bits_a, bits_b):
+    """Integer matrices whose products and sums FP64 holds come out exactly, as FP64 FMAs give them."""
+    import torch
+    V, rng = 1537, np.random.default_rng(5)
+    a, b = integers(V * 72, bits_a, rng), integers(72, bits_b, rng)
+    h = su3.Handle(0)
+    want = exact_and_bound(a, b)[0].astype(np.float64)
+    assert np.array_equal(run_form(h, a, b, su3.F64), want)
+    d, dev = su3.Desc(su3.F64, su3.FULL18, su3.AOS, V), torch.from_numpy(a).cuda()
+    at = np.ascontiguousarray(a.reshape(-1, 3, 3, 2).transpose(0, 2, 1, 3) * [1.0, -1.0]).reshape(-1)
+    out, w = torch.empty_like(dev), torch.empty(V * 24, dtype=torch.float64, device="cuda")
+    h.mult_op(su3.OP_AN, d, dev, b, d, out)
+    h.mat_vec(d, dev, b.reshape(4, 3, 3, 2)[:, :, 0].copy(), w)
+    h.sync()
+    assert np.array_equal(out.cpu().numpy(), exact_and_bound(at, b)[0].astype(np.float64))
+    assert np.array_equal(w.cpu().numpy(), want.reshape(-1, 3, 3, 2)[:, :, 0].reshape(-1))
+    h.close()
+
+
+@pytest.mark.parametrize("name", ["graded", "smooth", "one_direction", "wide"])
+def test_rows_do_not_depend_on_their_warp(name):
+    """Rows in fixed point, by FMAs and in part by each share warps: the same bits in any company."""
+    V, rng = 1537, np.random.default_rng(13)
+    a, b = family(name, V, rng)
+    h = su3.Handle(0)
+    c = run_form(h, a, b, su3.F64).reshape(V, 4, 18)
+    for j in range(4):  # another order of the sites, and the direction's links alone (others zero)
+        order = rng.permutation(V)
+        alone = np.zeros((V, 4, 18))
+        alone[:, j] = a.reshape(V, 4, 18)[order, j]
+        assert np.array_equal(run_form(h, alone.reshape(-1), b, su3.F64).reshape(V, 4, 18)[:, j], c[order, j])
     h.close()
 
 
@@ -127,7 +175,7 @@ def test_rows_in_every_layout(layout, ri, ro):
     h.close()
 
 
-@pytest.mark.parametrize("name", ["random", "graded", "real", "dyadic", "b_identity"])
+@pytest.mark.parametrize("name", ["random", "graded", "real", "dyadic", "small_terms", "wide", "b_small", "b_identity"])
 def test_adjacent_products(name):
     """a^dagger b, a v and a^dagger v: the same bounds, with a's columns (conjugated) as rows."""
     import torch
@@ -140,14 +188,14 @@ def test_adjacent_products(name):
     out = torch.empty_like(dev)
     h.mult_op(su3.OP_AN, d, dev, b, d, out)
     h.sync()
-    want, bound, _ = exact_and_bound(at.reshape(-1), b)
+    want, bound = exact_and_bound(at.reshape(-1), b)
     assert np.all(np.abs(out.cpu().numpy().astype(np.longdouble) - want) <= bound)
     v = b.reshape(4, 3, 3, 2)[:, :, 0].copy()  # the first column of each matrix
     for adjoint, rows in ((False, a), (True, at)):
-        want, _, chain = exact_and_bound(np.ascontiguousarray(rows).reshape(-1), b)
+        want, _ = exact_and_bound(np.ascontiguousarray(rows).reshape(-1), b)
         bv = np.zeros((4, 3, 3, 2))
         bv[:, :, 0] = v
-        _, bound, _ = exact_and_bound(np.ascontiguousarray(rows).reshape(-1), bv.reshape(-1))
+        _, bound = exact_and_bound(np.ascontiguousarray(rows).reshape(-1), bv.reshape(-1))
         w = torch.zeros(V * 24, dtype=torch.float64, device="cuda")
         h.mat_vec(d, dev, v, w, adjoint=adjoint)
         h.sync()
