@@ -392,8 +392,10 @@ __device__ __forceinline__ void link_mult(const Link<T>& a, const T (&bre)[9], c
 // to 0.79. S is estimated from below by two dot products of bytes, from |a| cut to 5 bits and |b| to 8.
 // An output real that does not pass, or is below 2^-26 of full scale (not normalised), is computed by
 // FP64 FMAs; so are all of a row whose reals are spread over more than 2^31 (any zero), not finite or
-// outside 2^-723 .. 2^677, and all rows when fix_b refuses b. Which way an output goes depends on its
-// row's and b's values only, so results are the same for every launch shape and layout.
+// outside 2^-723 .. 2^677, and all rows when fix_b refuses b. A warp does FMAs for the output reals
+// that any of its lanes needs and the sixth once for all, 36 of them at most: no mix of values takes
+// longer than FMAs throughout do. Which way an output goes depends on its row's and b's values only,
+// so results are the same for every launch shape and layout.
 // Measured (AOS, 48^4 sites, GB/s): FP64 FMAs alone 1,585; random SU(3) 5,128, 5,395 without the
 // gate; links exp(i e H) at e = 0.05 2,952; an identity or real a or b 1,575. The wide multiply-adds
 // and the other integer instructions share their issue, so they set the rate (364 instructions per
@@ -566,15 +568,19 @@ __device__ __forceinline__ unsigned fixed_row(const double (&are)[3], const doub
 }
 
 // A whole row c = a b (c as in fixed_row): its output reals in fixed point where that suits, the last
-// NAT and the others by FP64 FMAs. bj = b[j] in FP64.
+// NAT and the others by FP64 FMAs. bj = b[j] in FP64. The fixed-point part is run for every row, since a
+// branch around it would run the last NAT twice in a warp whose rows differ (one link of four the
+// identity, 2^21 sites: 1.78 ms with a branch, 1.53 so, 1.58 with FMAs throughout).
 template <int COLS, int NAT>
 __device__ __forceinline__ void row_f64(const double (&are)[3], const double (&aim)[3], const FixedB<COLS>& b,
                                         const double* bj, double (&c)[2 * COLS]) {
   constexpr int kOut = 2 * COLS - NAT;
   unsigned rest = ~0u;
-  FixedExps ex;
-  if (ex.take(are, aim, b.range)) {
+  if (b.range) {  // else b does not suit: the same for every thread
+    FixedExps ex;
+    const bool ok = ex.take(are, aim, b.range);
     rest = fixed_row<COLS, NAT>(are, aim, ex, b, c);
+    rest = ok ? rest : ~0u;
 #pragma unroll
     for (int o = kOut; o < 2 * COLS; ++o) c[o] = fma_output<COLS>(are, aim, bj, o);
   } else {
