@@ -182,7 +182,9 @@ LaunchCfg cfg_for(su3_handle* h, const su3_desc* d, const Form& f, bool adjacent
   auto it = h->cfgs.find(form_key(d, f.repr_out));
   if (it == h->cfgs.end() && f.repr_out != d->repr) it = h->cfgs.find(form_key(d));
   if (it != h->cfgs.end()) return it->second;
-  return adjacent ? default_adjacent_cfg(f) : default_cfg(f);
+  LaunchCfg c = adjacent ? default_adjacent_cfg(f) : default_cfg(f);
+  c.is_default = true;
+  return c;
 }
 
 // Validates an (a, c) descriptor pair into a Form.

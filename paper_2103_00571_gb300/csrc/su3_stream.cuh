@@ -480,24 +480,8 @@ static su3_status run_aos(const Form& f, const LaunchCfg& cfg_in, const void* a,
       }
     }
   }
-  // an array with fewer tiles than SMs: narrower tiles, in CTAs just wide enough for them, spread
-  // it over more SMs, so that its warps do not queue on a few SMs' pipes (every launch shape gives
-  // the same bits; this only shortens small launches)
-  if (f.n_sites > 0 && (f.n_sites + ts - 1) / ts < ctx.num_sms) {
-    long long t2 = (f.n_sites + ctx.num_sms - 1) / ctx.num_sms;
-    t2 = std::max(quantum, (t2 + quantum - 1) / quantum * quantum);
-    if (t2 < ts) {
-      ts = t2;
-      // FP64 in fixed point: one thread per output row while a tile's rows fit one CTA, since a whole
-      // link is a chain of three rows (per launch at 64 sites 5.8 -> 3.7 us, 1,000 sites 5.9 -> 4.3,
-      // 2,000 sites 5.3 -> 4.7; with more rows than threads, at 4,096 sites, 5.5 either way)
-      const bool split = kInPlace && Op::kRowSplit && Op::kFixCols > 0 && f.arith == SU3_ARITH_NATIVE &&
-                         ts * 4 * (Op::kNeOut / 3) <= 256;
-      if (split) cfg.threads_per_link = 3;
-      const long long items = ts * 4 * (cfg.threads_per_link == 1 ? 1 : (Op::kRowSplit ? Op::kNeOut / 3 : 1));
-      cfg.block = (int)std::min<long long>(split ? 256 : cfg.block, std::max<long long>(32, (items + 31) / 32 * 32));
-    }
-  }
+  spread_small(&cfg, &ts, f.n_sites, ctx.num_sms, quantum, Op::kRowSplit ? Op::kNeOut / 3 : 1,
+               kInPlace && Op::kRowSplit && Op::kFixCols > 0 && f.arith == SU3_ARITH_NATIVE);
   AosArgs<BA, Op::kFixCols> p;
   p.a = static_cast<const unsigned char*>(a);
   p.c = static_cast<unsigned char*>(c);
