@@ -108,7 +108,9 @@ typedef struct {
 
 typedef struct su3_handle su3_handle;
 
-/* Launch configuration of the streaming kernels (for the autotuner); 0 fields = default.
+/* Launch configuration of the streaming kernels (for the autotuner). Fields left 0 beside others take a
+ * shape that is the same for every size (AOS 128 threads, 4 stages, 2 CTAs per SM; AOSOA32/SOA 256
+ * threads, direct loads, 4 CTAs per SM); all 0 = back to the default, which is measured per form.
  * AOS always streams through shared memory (the staged kernel). AOSOA32 and SOA use the staged
  * kernel when stages is 2..8 and plain coalesced global loads when stages is 0 (their default).
  * At launch, an array with fewer tiles than SMs gets narrower tiles, in CTAs of at most `block` threads

@@ -360,7 +360,12 @@ su3_status set_cfg(su3_handle* h, const su3_desc* form, int repr_out, const su3_
   Form f;
   su3_status s = cfg_form(h, form, repr_out, &f);
   if (s != SU3_OK) return s;
-  LaunchCfg c = default_cfg(f);
+  if (!cfg->block && !cfg->tile_sites && !cfg->stages && !cfg->ctas_per_sm && !cfg->native_permille &&
+      !cfg->threads_per_link) {
+    h->cfgs.erase(form_key(form, repr_out));
+    return SU3_OK;
+  }
+  LaunchCfg c = general_cfg(f);
   if (cfg->block) c.block = cfg->block;
   if (cfg->tile_sites) c.tile_sites = cfg->tile_sites;
   if (cfg->stages) c.stages = cfg->stages;

@@ -55,6 +55,9 @@ inline int64_t link_bytes(int dtype, int repr) { return (int64_t)n_elem(repr) * 
 LaunchCfg default_cfg(const Form& f);
 // The same for su3_mult_op's a^dagger b and su3_mat_vec.
 LaunchCfg default_adjacent_cfg(const Form& f);
+// What su3_set_launch_cfg fills a partial configuration up with: independent of the array's size, and
+// shallow enough that any one field can be set beside it.
+LaunchCfg general_cfg(const Form& f);
 
 // An array with fewer tiles of *ts sites than SMs: narrower tiles (multiples of `quantum` sites), in
 // CTAs just wide enough for them, spread it over more SMs, so that its warps do not queue on a few SMs'

@@ -33,11 +33,23 @@ su3_status launch_selftest_wait(int limit_ms, const LaunchCtx& ctx) {
 
 // ---- host launchers -----------------------------------------------------------------------------
 
-// The AOS shape that suits every form somewhat: ~18 KB per tile for FP64 full sites, 9-18 KB for the
-// narrower ones, in 8 warps per SM. It divides small and middling arrays more evenly than larger tiles do.
-static LaunchCfg general_cfg(const Form& f) {
+// The shape that suits every form of a layout somewhat, whatever its size. AOS: ~18 KB per tile for FP64
+// full sites, 9-18 KB for the narrower ones, in 8 warps per SM, which divides small and middling arrays
+// more evenly than larger tiles do; AOSOA32 and SOA: direct loads, 1/2/4 links of 16/8/4-byte elements.
+LaunchCfg general_cfg(const Form& f) {
+  const bool aos = f.layout == SU3_LAYOUT_AOS;
   const int tile = (int)std::max<int64_t>(32, std::min<int64_t>(128, 18432 / std::max<int64_t>(f.a_stride, 1)));
-  return LaunchCfg{128, tile, 4, 2, 0, 1};
+  LaunchCfg c{128, tile, 4, 2, 0, 1};
+  if (!aos) c = LaunchCfg{256, f.dtype == SU3_F64 ? 1 : f.dtype == SU3_F32 ? 2 : 4, 0, 4, 0, 1};
+  if (f.arith == SU3_ARITH_HYBRID) {
+    c.native_permille = 125;
+    c.block = 256;  // 8 warps, one of them native
+    if (aos) {
+      c.tile_sites = 64;  // 256 links: one per thread and tile
+      c.stages = 3;       // two such CTAs fit in one SM's shared memory
+    }
+  }
+  return c;
 }
 
 // The shapes that measured best (block, sites per tile, stages, CTAs per SM, threads per link); GB/s at
@@ -80,20 +92,11 @@ static LaunchCfg measured_cfg(const Form& f) {
 LaunchCfg default_adjacent_cfg(const Form& f) { return f.dtype == SU3_F64 ? default_cfg(f) : general_cfg(f); }
 
 LaunchCfg default_cfg(const Form& f) {
+  if (f.arith == SU3_ARITH_HYBRID) return general_cfg(f);
   LaunchCfg c = measured_cfg(f);
   // a tile's sites may span 1 MiB of the array; wide strides keep tiles of 32 sites
   if (f.layout == SU3_LAYOUT_AOS)
     c.tile_sites = (int)std::min<int64_t>(c.tile_sites, std::max<int64_t>(32, (1 << 20) / std::max<int64_t>(f.a_stride, 1)));
-  c.native_permille = f.arith == SU3_ARITH_HYBRID ? 125 : 0;
-  if (f.arith == SU3_ARITH_HYBRID) {
-    c.block = 256;  // 8 warps, one of them native
-    c.threads_per_link = 1;
-    c.ctas_per_sm = f.layout == SU3_LAYOUT_AOS ? 2 : 4;
-    if (f.layout == SU3_LAYOUT_AOS) {
-      c.tile_sites = 64;  // 256 links: one per thread and tile
-      c.stages = 3;       // two such CTAs fit in one SM's shared memory
-    }
-  }
   return c;
 }
 

@@ -404,3 +404,26 @@ def test_measure_fp64_rate(h):
     assert 0.3 < tf < 3.0, tf
     with pytest.raises(su3.Su3Error):
         h.measure_fp64_rate(0)
+
+
+def test_partial_launch_cfg_does_not_depend_on_the_defaults():
+    """Fields left 0 take a fixed shape, not the measured default of the form and size."""
+    h = su3.Handle(0)
+    d = su3.Desc(su3.F64, su3.FULL18, su3.AOSOA32, 1000)
+    h.set_launch_cfg(d, block=256, tile_sites=64, stages=3)
+    assert h.get_launch_cfg(d)["ctas_per_sm"] == 4
+    small, large = (su3.Desc(su3.F32, su3.FULL18, su3.AOS, n) for n in (64, 1 << 22))
+    h.set_launch_cfg(small, ctas_per_sm=3)
+    assert h.get_launch_cfg(large) == dict(block=128, tile_sites=64, stages=4, ctas_per_sm=3, native_permille=0,
+                                           threads_per_link=1)
+    for dt in (su3.F64, su3.F32, su3.F16, su3.BF16):  # any one field beside the others' shape
+        for r in (su3.FULL18, su3.TWOROW12):
+            V = 2000
+            a, b = gen.lattice(3, V)
+            d = su3.Desc(dt, r, su3.AOS, V)
+            want = run_form(h, a, b, dt, r)
+            for cfg in (dict(block=32), dict(tile_sites=96), dict(stages=8), dict(ctas_per_sm=1), dict(threads_per_link=3)):
+                assert np.array_equal(run_form(h, a, b, dt, r, cfg=cfg), want), (dt, r, cfg)
+            h.set_launch_cfg(d)  # all 0: the default again
+            assert h.get_launch_cfg(d) == su3.Handle(0).get_launch_cfg(d)
+    h.close()
