@@ -203,3 +203,36 @@ def test_adjacent_products(name):
         err = np.abs(w.cpu().numpy().astype(np.longdouble) - pick(want))
         assert np.all(err <= pick(bound)), (name, adjoint)
     h.close()
+
+
+@pytest.mark.parametrize("tpl", [1, 3])
+def test_batched_families(tpl):
+    """Lattices whose b suits the form, does not, or has far exponents side by side in one batch: the bits
+    of the single-lattice kernel from every entry point."""
+    import ctypes
+    import torch
+    h, rng = su3.Handle(0), np.random.default_rng(17)
+    items, keep = [], []
+    for k, name in enumerate(FAMILIES):
+        V = 129 + 16 * k
+        a, b = family(name, V, rng)
+        dev = torch.from_numpy(a).cuda()
+        d = su3.Desc(su3.F64, su3.FULL18, su3.AOS, V)
+        c = torch.zeros_like(dev)
+        items.append(su3.BatchItem(d, dev.data_ptr(), c.data_ptr(), (ctypes.c_double * 72)(*b)))
+        keep.append((name, dev, c, run_form(h, a, b, su3.F64)))
+    h.set_batched_cfg(block=128 if tpl == 3 else 64, tile_sites=32, stages=3, ctas_per_sm=4, threads_per_link=tpl)
+    calls = [lambda: h.mult_batched(items, use_graph=False), lambda: h.mult_batched(items, use_graph=True),
+             lambda: h.mult_batched(items, use_graph=True)]
+    if tpl == 1:  # the static entry point has the default shape
+        arr, stream = (su3.BatchItem * len(items))(*items), torch.cuda.current_stream().cuda_stream
+        calls.append(lambda: su3.lib().su3_mult_batched_static(len(items), arr, ctypes.c_void_p(stream)))
+    for call in calls:
+        for _, _, c, _ in keep:
+            c.zero_()
+        call()
+        h.sync()
+        torch.cuda.synchronize()
+        for name, _, c, want in keep:
+            assert np.array_equal(c.cpu().numpy(), want), name
+    h.close()
