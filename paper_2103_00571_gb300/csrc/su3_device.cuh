@@ -257,6 +257,12 @@ template <typename A>
 struct BShared<A, 0> {
   A v[72];
 };
+template <typename A>
+struct BShared<A, 1> {  // one column: its limbs with either sign (FixedB<1>)
+  alignas(16) A v[72];
+  int fx[3][2][4][4];
+  unsigned mag[4][kFixMags];
+};
 template <class Op>
 using BSharedOf = BShared<typename Op::BArg, Op::kFixCols>;
 
@@ -265,15 +271,28 @@ template <class Op>
 __device__ __forceinline__ void load_b_op(const BMat<typename Op::BArg, Op::kFixCols>& b, BSharedOf<Op>* bsh, Op& op,
                                           int native_warps) {
   for (int i = threadIdx.x; i < 72; i += blockDim.x) bsh->v[i] = b.v[i];
-  if constexpr (Op::kFixCols > 0) {
+  if constexpr (Op::kFixCols == 1) {
+    for (int i = threadIdx.x; i < 3 * 4 * 2; i += blockDim.x) {  // element, direction, re or im
+      const int e = i >> 3, j = (i >> 1) & 3, c = 2 * (i & 1);
+      const long long x = ((long long)b.fix.fx[j][e][c] << 32) + b.fix.fx[j][e][c + 1];
+      for (int s = 0; s < 2; ++s) {
+        const long long v = s ? -x : x;
+        bsh->fx[e][s][j][c + 1] = (int)v;
+        bsh->fx[e][s][j][c] = (int)((v - (int)v) >> 32);
+      }
+    }
+  } else if constexpr (Op::kFixCols > 0) {
     for (int i = threadIdx.x; i < 4 * 9 * 4; i += blockDim.x) (&bsh->fx[0][0][0])[i] = (&b.fix.fx[0][0][0])[i];
+  }
+  if constexpr (Op::kFixCols > 0) {
     for (int i = threadIdx.x; i < 4 * kFixMags; i += blockDim.x) (&bsh->mag[0][0])[i] = (&b.fix.mag[0][0])[i];
   }
   __syncthreads();
   const int j = threadIdx.x & 3;
   op.init(bsh->v + 18 * j, native_warps);
   op.set_unit(b.unit);
-  if constexpr (Op::kFixCols > 0) op.set_fixed(b.fix, bsh->fx[j], bsh->mag[j], j);
+  if constexpr (Op::kFixCols == 1) op.set_fixed(b.fix, bsh->fx[0][0][j], bsh->mag[j], j);
+  else if constexpr (Op::kFixCols > 0) op.set_fixed(b.fix, bsh->fx[j], bsh->mag[j], j);
 }
 
 // ---- the link product -------------------------------------------------------------------------
@@ -403,7 +422,9 @@ __device__ __forceinline__ void link_mult(const Link<T>& a, const T (&bre)[9], c
 // b is read from shared memory for each row: in registers 4,869, at 124 of them instead of 112. S in FP32,
 // on the idle half of the FP32 pipe: 4,739.
 
-// b[j] (or v[j]) of one thread in fixed point, in memory: element e = 3*m + l (COLS 3) or m (COLS 1).
+// b[j] (or v[j]) of one thread in fixed point, in memory. COLS 3: element e = 3*m + l at limbs[e]. COLS 1:
+// element m at limbs[8*m], its negative at limbs[8*m + 4] (the four directions' side by side, so that
+// the addresses of a warp's load fall into different banks).
 template <int COLS>
 struct FixedB {
   const int4* limbs;  // (re_hi, re_lo, im_hi, im_lo)
@@ -489,6 +510,48 @@ __device__ __forceinline__ double fma_output(const double (&are)[3], const doubl
   return c;
 }
 
+// a's real x in fixed point without its sign, d binary orders below its row's largest: hi * 2^32 + lo, hi
+// of 29 bits.
+__device__ __forceinline__ void cut_real(double x, int d, unsigned lead, unsigned& hi, unsigned& lo) {
+  const unsigned l = (unsigned)__double2loint(x);
+  const unsigned m = ((unsigned)__double2hiint(x) & 0xfffffu) | lead;
+  const unsigned w = __funnelshift_l(l, m, 8);
+  hi = w >> d;
+  lo = __funnelshift_r(l << 8, w, d);
+}
+
+// The set of output reals (bit 2*l + im) that do not pass the gate; `mag`: |re| of a's three elements,
+// then |im|, 29 bits each.
+template <int COLS, int NAT>
+__device__ __forceinline__ unsigned small_outputs(const unsigned (&mag)[6], const uint4* mags) {
+  constexpr int kOut = 2 * COLS - NAT;
+  // |re|, |im| of elements 0 and 1, then of 2, in bytes of 1/32 of full scale; im's sums take
+  // them the other way round
+  const unsigned r01 = __byte_perm(__byte_perm(mag[0], mag[3], 0x0073), __byte_perm(mag[1], mag[4], 0x0073), 0x5410);
+  const unsigned r2 = __byte_perm(mag[2], mag[5], 0x0073);  // b's bytes 2 and 3 are 0 here
+  const unsigned i01 = __byte_perm(r01, 0, 0x2301), i2 = __byte_perm(r2, 0, 0x2301);
+  unsigned bm[(2 * COLS + 3) / 4 * 4], rest = 0;
+#pragma unroll
+  for (int i = 0; i < (2 * COLS + 3) / 4; ++i) {
+    const uint4 v = mags[i];
+    bm[4 * i] = v.x;
+    bm[4 * i + 1] = v.y;
+    bm[4 * i + 2] = v.z;
+    bm[4 * i + 3] = v.w;
+  }
+#pragma unroll
+  for (int o = kOut - 1; o >= 0; --o) {
+    const unsigned sum = __dp4a(o & 1 ? i2 : r2, bm[o | 1], 0u - kFixMinSum);
+    rest = __funnelshift_l(__dp4a(o & 1 ? i01 : r01, bm[o & ~1], sum), rest, 1);  // its sign
+  }
+  return rest;
+}
+
+// T from H, X and Y.
+__device__ __forceinline__ long long sum_limbs(long long h, long long x, long long y) {
+  return h + (long long)((unsigned long long)x >> 32) + (long long)((unsigned long long)y >> 32);
+}
+
 // The output reals of a row but for the last NAT: c[2*l] = re and c[2*l + 1] = im of sum_m a[m] b[m][l],
 // l < COLS. Returns the set (bit 2*l + im) of those that FP64 FMAs have to do instead.
 template <int COLS, int NAT>
@@ -500,12 +563,12 @@ __device__ __forceinline__ unsigned fixed_row(const double (&are)[3], const doub
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
     const double x = q < 3 ? are[q % 3] : aim[q % 3];
-    const int h = __double2hiint(x);
-    const unsigned l = (unsigned)__double2loint(x);
-    const unsigned m = ((unsigned)h & 0xfffffu) | b.k.lead;
-    const unsigned w = __funnelshift_l(l, m, 8), s = (unsigned)(h >> 31);
-    mag[q] = w >> ex.d[q];
-    unsigned vh = mag[q] ^ s, vl = __funnelshift_r(l << 8, w, ex.d[q]) ^ s;
+    unsigned vh, vl;
+    cut_real(x, ex.d[q], b.k.lead, vh, vl);
+    mag[q] = vh;
+    const unsigned s = (unsigned)(__double2hiint(x) >> 31);
+    vh ^= s;
+    vl ^= s;
     asm("{sub.cc.u32 %0, %0, %2; subc.u32 %1, %1, %2;}" : "+r"(vl), "+r"(vh) : "r"(s));
     ah[q] = (int)(vh + (vl >> 31));
     al[q] = (int)vl;
@@ -515,30 +578,9 @@ __device__ __forceinline__ unsigned fixed_row(const double (&are)[3], const doub
       nl[q - 3] = (int)vl;
     }
   }
-  // the gate: |re|, |im| of elements 0 and 1, then of 2, in bytes of 1/32 of full scale; im's sums take
-  // them the other way round
-  const unsigned r01 = __byte_perm(__byte_perm(mag[0], mag[3], 0x0073), __byte_perm(mag[1], mag[4], 0x0073), 0x5410);
-  const unsigned r2 = __byte_perm(mag[2], mag[5], 0x0073);  // b's bytes 2 and 3 are 0 here
-  const unsigned i01 = __byte_perm(r01, 0, 0x2301), i2 = __byte_perm(r2, 0, 0x2301);
-  unsigned bm[(2 * COLS + 3) / 4 * 4], rest = 0;
-#pragma unroll
-  for (int i = 0; i < (2 * COLS + 3) / 4; ++i) {
-    const uint4 v = b.mags[i];
-    bm[4 * i] = v.x;
-    bm[4 * i + 1] = v.y;
-    bm[4 * i + 2] = v.z;
-    bm[4 * i + 3] = v.w;
-  }
-#pragma unroll
-  for (int o = kOut - 1; o >= 0; --o) {
-    const unsigned sum = __dp4a(o & 1 ? i2 : r2, bm[o | 1], 0u - kFixMinSum);
-    rest = __funnelshift_l(__dp4a(o & 1 ? i01 : r01, bm[o & ~1], sum), rest, 1);  // its sign
-  }
+  const unsigned rest = small_outputs<COLS, NAT>(mag, b.mags);
   const unsigned base = ((0x7ffu - (unsigned)ex.e0) << 20) + b.kb;
   unsigned bad = ex.spread();
-  auto sum3 = [](long long h, long long u, long long v) {
-    return h + (long long)((unsigned long long)u >> 32) + (long long)((unsigned long long)v >> 32);
-  };
 #pragma unroll
   for (int l = 0; l < COLS; ++l) {
     // re and im together: six independent chains of multiply-adds
@@ -561,9 +603,48 @@ __device__ __forceinline__ unsigned fixed_row(const double (&are)[3], const doub
         yi = mad_wide(al[3 + m], w.x, yi);
       }
     }
-    c[2 * l] = fixed_to_f64(sum3(hr, xr, yr), base, bad);
-    if (2 * l + 1 < kOut) c[2 * l + 1] = fixed_to_f64(sum3(hi, xi, yi), base, bad);
+    c[2 * l] = fixed_to_f64(sum_limbs(hr, xr, yr), base, bad);
+    if (2 * l + 1 < kOut) c[2 * l + 1] = fixed_to_f64(sum_limbs(hi, xi, yi), base, bad);
   }
+  return bad & ~31u ? ~0u : rest;
+}
+
+// The same for one column, c[0] = re and c[1] = im: a's limbs without their signs, which choose b's
+// instead. With two outputs a row, six sign changes and three negations cost more than the loads (a v
+// at L=48 5,566 -> 6,158 GB/s, a^dagger v 5,246 -> 5,695; with three columns the loads cost more, 5,094 ->
+// 4,808).
+__device__ __forceinline__ unsigned fixed_row(const double (&are)[3], const double (&aim)[3], const FixedExps& ex,
+                                              const FixedB<1>& b, double (&c)[2]) {
+  unsigned mag[6], low[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) cut_real(q < 3 ? are[q % 3] : aim[q % 3], ex.d[q], b.k.lead, mag[q], low[q]);
+  const unsigned rest = small_outputs<1, 0>(mag, b.mags);
+  const unsigned base = ((0x7ffu - (unsigned)ex.e0) << 20) + b.kb;
+  unsigned bad = ex.spread();
+  long long hr = b.k.hbias, xr = b.k.xbias, yr = b.k.xbias, hi = b.k.hbias, xi = b.k.xbias, yi = b.k.xbias;
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    const int sr = (__double2hiint(are[m]) >> 31) & 4, si = (__double2hiint(aim[m]) >> 31) & 4;
+    const int4 w = b.limbs[8 * m + sr];                                                   // b with re's sign
+    const int2 u = reinterpret_cast<const int2*>(b.limbs)[2 * (8 * m + (si ^ 4)) + 1];  // im of b with -im's
+    const int2 v = reinterpret_cast<const int2*>(b.limbs)[2 * (8 * m + si)];              // re of b with im's
+    const int rh = (int)(mag[m] + (low[m] >> 31)), rl = (int)low[m];
+    const int ih = (int)(mag[3 + m] + (low[3 + m] >> 31)), il = (int)low[3 + m];
+    hr = mad_wide(rh, w.x, hr);
+    hr = mad_wide(ih, u.x, hr);
+    xr = mad_wide(rh, w.y, xr);
+    xr = mad_wide(ih, u.y, xr);
+    yr = mad_wide(rl, w.x, yr);
+    yr = mad_wide(il, u.x, yr);
+    hi = mad_wide(rh, w.z, hi);
+    hi = mad_wide(ih, v.x, hi);
+    xi = mad_wide(rh, w.w, xi);
+    xi = mad_wide(ih, v.y, xi);
+    yi = mad_wide(rl, w.z, yi);
+    yi = mad_wide(il, v.x, yi);
+  }
+  c[0] = fixed_to_f64(sum_limbs(hr, xr, yr), base, bad);
+  c[1] = fixed_to_f64(sum_limbs(hi, xi, yi), base, bad);
   return bad & ~31u ? ~0u : rest;
 }
 
@@ -579,7 +660,8 @@ __device__ __forceinline__ void row_f64(const double (&are)[3], const double (&a
   if (b.range) {  // else b does not suit: the same for every thread
     FixedExps ex;
     const bool ok = ex.take(are, aim, b.range);
-    rest = fixed_row<COLS, NAT>(are, aim, ex, b, c);
+    if constexpr (COLS == 1) rest = fixed_row(are, aim, ex, b, c);
+    else rest = fixed_row<COLS, NAT>(are, aim, ex, b, c);
     rest = ok ? rest : ~0u;
 #pragma unroll
     for (int o = kOut; o < 2 * COLS; ++o) c[o] = fma_output<COLS>(are, aim, bj, o);
@@ -831,7 +913,7 @@ struct MatVecOp {  // w[k] = sum_m a[k][m] v[m]   (ADJ: sum_m conj(a[m][k]) v[m]
 // The same for FP64 storage, rows in fixed point (fixed_row): row k of a^dagger b is the conjugate of
 // a's column k times b, and an element of a v is a's row k times the one column v (all in fixed point:
 // with one of six on the FP64 pipe a^dagger v measured 9 % slower). At L=48, FP64 FMAs before:
-// a^dagger b 1,568 -> 4,836 GB/s, a v 2,960 -> 5,566, a^dagger v 2,950 -> 5,246 (the products' launch shape).
+// a^dagger b 1,568 -> 4,852 GB/s, a v 2,960 -> 6,158, a^dagger v 2,950 -> 5,695 (the products' launch shape).
 template <>
 struct AnOp<kF64> {
   using V = double2;
