@@ -137,7 +137,7 @@ def candidates(desc, out=None):
     if desc.layout == B.AOS:
         site = B.link_bytes(desc.dtype, desc.repr) * 4  # shared-memory tiles are packed whatever the stride
         out = []  # threads_per_link 3 = one thread per output row
-        for block, stages, cps, tpl in itertools.product((64, 128, 192, 256), (3, 4, 6), (1, 2, 3, 4, 6), (1, 3)):
+        for block, stages, cps, tpl in itertools.product((64, 128, 192, 256), (2, 3, 4, 6), (1, 2, 3, 4, 6), (1, 3)):
             # tiles of ~9/18/36 KB, and tiles of exactly one or two links per thread
             sizes = sorted({max(8, tb // site) for tb in (9216, 18432, 36864)} | {block // 4, block // 2})
             for ts in sizes:
