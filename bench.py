@@ -481,10 +481,12 @@ def run_native(args, world, rank, local):
     # roofline of the dominant kernel (the FP64 AoS kernel is the whole step); its template's
     # threads per link: 1, or 3 when the launch splits links into rows
     tpl = 3 if h.get_launch_cfg_for(d64, dc)["threads_per_link"] == 3 else 1
-    # The FP64 product's peak, TFLOP/s by the paper's count: the FP64 pipe's 2 FMA per clock and SM beside
-    # the integer units' 32 wide multiply-adds, of which 18 make the 6 FMAs of one output real
-    fp64_peak = sms * (2 * 2 + 32 / 18 * 6 * 2) * sm_max * 1e6 / 1e12
+    # An upper bound of the FP64 product's rate, TFLOP/s by the paper's count: its wide multiply-adds (18 for
+    # an output real, five or six of a row's six) back to back at 32 per clock and SM, the FP64 pipe's share
+    # beside them. The other integer instructions share the multiply-adds' issue, so it cannot be reached.
     flop_site = flop_per_site(d64.repr, dc.repr)
+    rows_site = 12 if dc.repr == su3.FULL18 else 8
+    fp64_peak = sms * 32 * flop_site / (18 * (5 if d64.repr == dc.repr else 6) * rows_site) * sm_max * 1e6 / 1e12
     fp64_share = 1 / 6 if d64.repr == dc.repr else 192 / flop_site  # of the flops, on the FP64 pipe
     achieved_tf = flop_site * V / (per_launch_ms * 1e-3) / 1e12
     achieved_gbs = bytes_per_step / (per_launch_ms * 1e-3) / 1e9
@@ -512,9 +514,9 @@ def run_native(args, world, rank, local):
         roofline = {"bound": "alu", "achieved": round(achieved_tf, 4), "peak": round(fp64_peak, 4),
                     "unit": "TFLOP/s", "frac": round(achieved_tf / fp64_peak, 4), "traffic": traffic,
                     "kernel": "su3_aos_kernel<NativeOp<F64,%s>, %d, AOS, %s>" % (ops, tpl, padded),
-                    "peak_source": "%d SMs (this device) x %.0f MHz (max SM clock) x (FP64 pipe 2 DFMA/clk x 2 flop + "
-                                   "integer units 32 wide multiply-adds/clk, 18 for the 12 flop of an output real)"
-                                       % (sms, sm_max),
+                    "peak_source": "%d SMs (this device) x %.0f MHz (max SM clock) x 32 wide multiply-adds/clk, 18 for an "
+                                   "output real in fixed point; an upper bound: the other integer instructions share "
+                                   "their issue" % (sms, sm_max),
                     "peak_measured": round(fp64_measured, 4) if fp64_measured else None,
                     "frac_of_measured": round(achieved_tf * fp64_share / fp64_measured, 4) if fp64_measured else None,
                     "peak_measured_source": "the FP64 pipe alone, and the share of the flops that it does (one output "
