@@ -42,7 +42,7 @@ __device__ __forceinline__ double2 ld_stream_16(const void* p) {
 }
 
 template <class Op>
-__global__ void __launch_bounds__(256) su3_host_kernel(const __grid_constant__ HostArgs<typename Op::BArg, Op::kFixCols> p) {
+__global__ void __launch_bounds__(256, Op::kMinCtas ? 2 : 0) su3_host_kernel(const __grid_constant__ HostArgs<typename Op::BArg, Op::kFixCols> p) {
   using V = typename Op::V;
   constexpr int NE_IN = Op::kNeIn, NE_OUT = Op::kNeOut;
   constexpr bool kInPlace = (NE_OUT == NE_IN);
