@@ -404,7 +404,7 @@ __device__ __forceinline__ void link_mult(const Link<T>& a, const T (&bre)[9], c
 // as a rule by 0.5. Limbs of zero make no error: products of few enough bits for FP64 FMAs to be
 // exact (integers, as a rule) are exact here too.
 // The 3.7 units do not shrink with the terms, so every output real passes a gate: the sum S of its six
-// |a||b| must be 1/16 of full scale, and is not in 1 of 10^5 of random SU(3) matrices. Then 3.7 units
+// |a||b| must be 1/16 of full scale (by the estimate below it is not for 3 of 10^5 with random SU(3) matrices). Then 3.7 units
 // are at most 1.9 * 2^-53 S, and the output is off by at most 2^-53 |c| + 1.9 * 2^-53 S, against 6 *
 // 2^-53 S for six FMAs; over the matrices tried (random and near the identity, reals spread over
 // up to 31 binary orders, integers) at most 1.6 * 2^-53 S against 4.7, r.m.s. 0.24 to 0.42 against 0.45
@@ -415,11 +415,11 @@ __device__ __forceinline__ void link_mult(const Link<T>& a, const T (&bre)[9], c
 // that any of its lanes needs and the sixth once for all, 36 of them at most: no mix of values takes
 // longer than FMAs throughout do. Which way an output goes depends on its row's and b's values only,
 // so results are the same for every launch shape and layout.
-// Measured (AOS, 48^4 sites, GB/s): FP64 FMAs alone 1,585; random SU(3) 5,128, 5,395 without the
-// gate; links exp(i e H) at e = 0.05 2,952; an identity or real a or b 1,575. The wide multiply-adds
+// Measured (AOS, 48^4 sites, GB/s): FP64 FMAs alone 1,585; random SU(3) 5,099-5,128, 5,395 without the
+// gate; links exp(i e H) at e = 0.05 2,982; an identity or real a or b 1,575. The wide multiply-adds
 // and the other integer instructions share their issue, so they set the rate (364 instructions per
 // row, 90 of them wide multiply-adds). 4 of 18 output reals on the FP64 pipe instead of 3: 4,916.
-// b is read from shared memory for each row: in registers 4,869, at 124 of them instead of 112. S in FP32,
+// b is read from shared memory for each row: in registers 4,869, at 124 of them instead of 108. S in FP32,
 // on the idle half of the FP32 pipe: 4,739.
 
 // b[j] (or v[j]) of one thread in fixed point, in memory. COLS 3: element e = 3*m + l at limbs[e]. COLS 1:

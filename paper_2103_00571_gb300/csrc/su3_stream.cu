@@ -71,8 +71,8 @@ static LaunchCfg measured_cfg(const Form& f) {
   }
   if (f.dtype == SU3_F64 && f.arith == SU3_ARITH_NATIVE) {
     if (two_out) return cfg(128, 48, 3, 4, 3);  // 4,977: 16 warps, rows as work items
-    if (two_in) return cfg(64, 24, 2, 6, 1);    // 2,925: 12 warps of 154 registers; with three stages they do not fit
-    return cfg(128, 32, 3, 4, 1);               // 5,094: 16 warps of 110 registers
+    if (two_in) return cfg(64, 24, 2, 6, 1);    // 3,019: 12 warps of 154 registers; with three stages they do not fit
+    return cfg(128, 32, 3, 4, 1);               // 5,094: 16 warps of 108 registers
   }
   if (f.dtype == SU3_F64) {  // FP32 pairs
     if (two_in) return cfg(128, 64, 3, 3, 1);                   // 5,683 (3,758); to full 4,430 (3,194)

@@ -102,7 +102,7 @@ __device__ __forceinline__ int tile_link_base(int q) {
 // maps; otherwise `maps` is read only by SOA tensor copies. One instantiation per PADDED value, so
 // the packed kernels keep their own code.
 // Launch bounds: a stated minimum of two CTAs per SM lets the compiler use up to 128 registers for its
-// schedule (FP64 rows in fixed point: 110 instead of 76, 5,098 instead of 4,755 GB/s at L=48; two-row 4,863
+// schedule (FP64 rows in fixed point: 108 instead of 76, 5,098 instead of 4,755 GB/s at L=48; two-row 4,863
 // instead of 4,484). The other ops run faster, or as fast, with the registers it takes by itself
 // (0: not stated).
 template <class Op, int TPL, int LAYOUT, bool PADDED>
